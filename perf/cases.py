@@ -104,7 +104,7 @@ def draw(rng):
                 continue
             return c
         if kind == "reduce":
-            c = dict(kind=kind, nt=64, nc=spread(60, 768), nb=rng.randint(6, 12),
+            c = dict(kind=kind, nt=64, nc=spread(60, 768, 2), nb=rng.randint(6, 12),
                      spacing="log", flagged=rng.random() < 0.5, n_k1=rng.randint(6, 16),
                      n_mu=rng.randint(3, 8), n_t=rng.randint(3, 8), lmax=rng.choice([0, 2, 4]),
                      n_cyl=rng.randint(5, 24))
