@@ -817,16 +817,18 @@ bs_status bs_bs_cylindrical(bs_plan p, const double *b3d, const double *kpar_hos
   if (st != BS_OK) return st;
   const int nc = p->nc, npl = (int)p->clos.size();
   // bins along one axis: q = (number of edges <= k_par) - 1, decided on the host
-  std::vector<int> &tab = p->cyl_tab;  // qa [nc], then seg [n] as (start, end)
-  tab.assign((size_t)nc + 2 * n, 0);
+  // qa [nc], then seg [n] as (start, end), read as int2: from an even index on
+  std::vector<int> &tab = p->cyl_tab;
+  const int so = (nc + 1) & ~1;
+  tab.assign((size_t)so + 2 * n, 0);
   std::vector<long long> na(n, 0);
   for (int c = 0; c < nc; ++c) {
     int q = (int)(std::upper_bound(edges_host, edges_host + n + 1, kpar_host[c]) - edges_host) - 1;
     if (q >= n) q = -1;
     tab[c] = q;
     if (q >= 0) {
-      if (na[q]++ == 0) tab[nc + 2 * q] = c;
-      tab[nc + 2 * q + 1] = c + 1;
+      if (na[q]++ == 0) tab[so + 2 * q] = c;
+      tab[so + 2 * q + 1] = c + 1;
     }
   }
   std::vector<long long> &cnt = p->cyl_cnt;
@@ -850,7 +852,7 @@ bs_status bs_bs_cylindrical(bs_plan p, const double *b3d, const double *kpar_hos
     MONO_CUDA(cudaMemsetAsync(sum_dev, 0, (size_t)batch * rest * sizeof(double), s));
   }
   const dim3 grid(npl, batch, 2);  // two row ranges per plane
-  const int2 *seg = reinterpret_cast<const int2 *>(dtab + nc);
+  const int2 *seg = reinterpret_cast<const int2 *>(dtab + so);
   if (nc <= kCylThreads)
     k_bs_cylindrical<1><<<grid, kCylThreads, sm, s>>>(b3d, bst, nc, n, dtab, seg, sums);
   else if (nc <= 2 * kCylThreads)

@@ -149,7 +149,8 @@ void compute_layout(bs_plan p) {
   // monopole binning constants: FP64 kperp [nb], kpar [nc]; FP32 kperp, kpar,
   // squared k1 edges [<= 1025], mu and t thresholds [<= 1025 each]
   L.mono = take(((size_t)p->nb + p->nc) * 12 + (size_t)3 * 1025 * 4 + 64);
-  L.cyl = take(((size_t)p->nc + 2 * 64) * sizeof(int));  // cylindrical bins (n <= 64)
+  // cylindrical bins: qa [nc], then (at an even index) seg [n <= 64] as int2
+  L.cyl = take(((size_t)p->nc + 1 + 2 * 64) * sizeof(int));
   // error bound: per-field norms (max |F|, ||F||_2, ||F||_3) of every level, and
   // the ring-triple table (i, j, l, level)
   size_t nfield_all = 0;

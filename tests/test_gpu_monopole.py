@@ -186,6 +186,28 @@ def test_monopole_more_realisations_than_one_launch_holds():
     plan.close()
 
 
+@pytest.mark.parametrize("nc", [9, 33, 257])
+def test_cylindrical_binning_odd_channels(nc):
+    """Odd channel counts: the bin ranges after the per-index table are read as pairs,
+    which have to start on an even word."""
+    torch = _torch()
+    import paper_2506_10526_gb300 as bs
+    edges = [1.0, 3.0, 5.0]
+    plan = bs.Plan(16, nc, edges)
+    plan.grid_load(torch.zeros((1, nc, 16, 16), dtype=torch.complex64, device="cuda"))
+    b3h = np.random.default_rng(nc).normal(size=(1, plan.n_closable, nc, nc))
+    kpar = mo.kpar_axis(nc)
+    ke = np.linspace(-0.8 * kpar.max(), 0.9 * kpar.max(), 6)
+    sums, cnt = plan.bs_cylindrical(torch.from_numpy(b3h).cuda(), kpar, ke)
+    torch.cuda.synchronize()
+    s_o, c_o = mo.bs_cylindrical(b3h, kpar, ke)
+    np.testing.assert_array_equal(cnt.cpu().numpy(), c_o)
+    scale = np.abs(b3h).max() * np.maximum(c_o, 1)
+    assert np.all(np.abs(sums.cpu().numpy() - s_o) <= 1e-12 * scale)
+    plan.close()
+
+
+
 @pytest.mark.parametrize("nc", [1000, 2160])  # 8 and 16 columns per thread; 2160: 4 delay rows per CTA
 def test_cylindrical_binning_wide_rows(nc):
     torch = _torch()
