@@ -29,16 +29,9 @@
 // The bin of a sample depends only on the geometry (k tables, edges, bin
 // counts, closable ring triples), not on the values, so the plan keeps an
 // int16 table of the bins of every sample and rebuilds it only when the
-// geometry changes (k_mono_bins: one thread per sample).  The summing kernel
-// (k_mono_sum) then streams the table and the values with coalesced loads:
-// each warp walks a contiguous range 32 samples at a time; when all 32 share
-// the warp's running bin each lane adds its value to its own per-realisation
-// running sums, which are reduced across the warp and flushed to the CTA's
-// shared-memory histogram only when the bin changes (neighbouring delay modes
-// mostly share a bin); mixed groups add per lane.  One FP64 add per sample
-// and realisation remains: the GB300 FP64 rate (about 0.5e12 adds/s
-// measured), not HBM, is what bounds the kernel.  The CTA adds its non-empty
-// bins to the global sums with FP64 atomics.
+// geometry changes (k_mono_bins: one thread per sample).  The summing kernels
+// then stream the table and the values with coalesced loads; the CTA adds its
+// non-empty bins to the global sums with FP64 atomics.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -70,7 +63,8 @@ struct MonoArgs {
   const double *kpar64;  // [nc]
   const float *thr;      // E [n_k1 + 1] | cmu [n_mu + 1] | ct [n_t + 1]
   int nc, n_k1, n_mu, n_t, nbin;
-  int chunk;             // samples per CTA, a multiple of 256 (nc^2 < 2^31)
+  int chunk;             // rows of a summing warp's range (mono_split)
+  int mirror;            // multipoles: kpar is antisymmetric, samples go in pairs
   int model;
   double f2, p_amp, p_half;  // 2 f_NG, amplitude, p_index / 2
   double *sums;          // [batch_total][nbin]
@@ -139,11 +133,54 @@ __global__ void __launch_bounds__(kThreads) k_mono_bins(const MonoArgs a, long l
   }
 }
 
-constexpr int kSumUnroll = 8;  // groups of 32 samples loaded ahead per warp
+// A summing warp owns 32 neighbouring columns (delay index b) of one plane and
+// walks down a range of rows (delay index a): unit u of a plane is column group
+// u % ncw, row range u / ncw.  The loads of a row are coalesced, and a lane's
+// samples change bin slowly (a bin is a curve-bounded patch of the (a, b)
+// plane), so each lane keeps the running sums of its own bin and adds them to the
+// CTA's histogram only when its bin changes.  Walking along rows with one bin
+// for the whole warp, nearly every group of 32 samples was mixed where the bins
+// are narrow along b, and went sample by sample through FP64 shared-memory
+// atomics (compare-and-swap loops): 3.34 ms for 216 planes of 768^2 (12 x 5 x 5
+// bins) against 0.43 ms now, 2.9 TB/s of bins and values (the FP64 adds alone
+// take 0.24 ms).
+//
+// Adds x[0..NX) of the lanes in `who` (a ballot; each lane's own bin `cur`) to the
+// histogram rows hs[k * nbin + cur], and their counts.  Called by the whole
+// warp.  Lanes that close the same bin are summed by shuffles first: their
+// atomics would serialise on one address.
+template <int NX>
+__device__ __forceinline__ void flush_lanes(unsigned who, int cur, const double *x, unsigned cnt,
+                                            int nx, int nbin, double *hs, unsigned *hc, int lane) {
+  while (who) {
+    const int bin = __shfl_sync(0xffffffffu, cur, __ffs(who) - 1);
+    const bool mine = ((who >> lane) & 1u) && cur == bin;
+    const unsigned grp = __ballot_sync(0xffffffffu, mine);
+    who &= ~grp;
+    if (__popc(grp) > 2) {
+      unsigned c = mine ? cnt : 0u;
+      for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+      if (lane == 0) atomicAdd(hc + bin, c);
+#pragma unroll
+      for (int k = 0; k < NX; ++k) {
+        if (k >= nx) break;
+        double v = mine ? x[k] : 0.0;
+        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) atomicAdd(hs + (size_t)k * nbin + bin, v);
+      }
+    } else if (mine) {
+      atomicAdd(hc + bin, cnt);
+#pragma unroll
+      for (int k = 0; k < NX; ++k)
+        if (k < nx) atomicAdd(hs + (size_t)k * nbin + bin, x[k]);
+    }
+  }
+}
 
 template <int NB>  // realisations per launch held in registers (a.nbatch <= NB)
 __global__ void __launch_bounds__(kThreads) k_mono_sum(const MonoArgs a,
                                                        const int16_t *__restrict__ bins) {
+  constexpr int UR = NB == 1 ? 8 : NB == 2 ? 4 : 2;  // rows loaded ahead
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double *hs = reinterpret_cast<double *>(smem_raw);                             // [nbatch][nbin]
   unsigned *hc = reinterpret_cast<unsigned *>(hs + (size_t)a.nbatch * a.nbin);  // [nbin]
@@ -153,88 +190,59 @@ __global__ void __launch_bounds__(kThreads) k_mono_sum(const MonoArgs a,
   __syncthreads();
   const int nb = a.model ? 1 : a.nbatch;
   const int i = a.rings[3 * p], j = a.rings[3 * p + 1], l = a.rings[3 * p + 2];
-  const int n = a.nc * a.nc;
-  const int c0 = blockIdx.x * a.chunk, c1 = min(n, c0 + a.chunk);
-  // this warp's contiguous range
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kThreads / 32;
-  const int per = ((c1 - c0 + nw - 1) / nw + 31) / 32 * 32;
-  const int w0 = min(c1, c0 + warp * per), w1 = min(c1, w0 + per);
-  const int16_t *bp = bins + (long long)p * n;
-  const double *vb = a.b3d ? a.b3d + (long long)a.b0 * a.bstride + (long long)p * n : nullptr;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int unit = blockIdx.x * (kThreads / 32) + warp, ncw = (a.nc + 31) / 32;
+  const int ib = (unit % ncw) * 32 + lane;
+  const int ia0 = min(a.nc, (unit / ncw) * a.chunk), ia1 = min(a.nc, ia0 + a.chunk);
+  const bool on = ib < a.nc;
+  const long long off = (long long)p * a.nc * a.nc + ib;
+  const int16_t *bp = bins + off;
+  const double *vb = a.b3d ? a.b3d + (long long)a.b0 * a.bstride + off : nullptr;
 
-  // The warp's running bin (uniform across the warp) and count; each lane keeps
-  // its own per-realisation running sums (one FP64 add per sample: the FP64 rate
-  // of the part bounds this kernel), reduced across the warp only when flushed.
   int cur = -1;
   unsigned cnt = 0;
   double run[NB];
 #pragma unroll
   for (int b = 0; b < NB; ++b) run[b] = 0.0;
-  auto flush = [&]() {
-    if (cur >= 0) {
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        if (b >= nb) break;
-        double x = run[b];
-        for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) atomicAdd(hs + (size_t)b * a.nbin + cur, x);
-      }
-      if (lane == 0) atomicAdd(hc + cur, cnt);
-    }
-    cnt = 0;
-#pragma unroll
-    for (int b = 0; b < NB; ++b) run[b] = 0.0;
-  };
-  for (int g0 = w0; g0 < w1; g0 += 32 * kSumUnroll) {
-    int q[kSumUnroll];
-    double v[kSumUnroll][NB];
+  for (int g0 = ia0; g0 < ia1; g0 += UR) {
+    int q[UR];
+    double v[UR][NB];
     // bins and values are loaded together (no load waits on another)
 #pragma unroll
-    for (int u = 0; u < kSumUnroll; ++u) {
-      const int e = g0 + 32 * u + lane;
-      q[u] = e < w1 ? (int)bp[e] : -1;
+    for (int u = 0; u < UR; ++u) {
+      const int ia = g0 + u;
+      const bool live = on && ia < ia1;
+      const long long e = (long long)ia * a.nc;
+      q[u] = live ? (int)bp[e] : -1;
       if (q[u] >= 0 && !BS_CHK(q[u], a.nbin, 41)) q[u] = -1;  // a bin outside the histogram
 #pragma unroll
       for (int b = 0; b < NB; ++b)
-        v[u][b] = (!a.model && b < nb && e < w1) ? __ldg(vb + (long long)b * a.bstride + e) : 0.0;
+        v[u][b] = (!a.model && b < nb && live) ? __ldg(vb + (long long)b * a.bstride + e) : 0.0;
     }
     if (a.model) {
 #pragma unroll
-      for (int u = 0; u < kSumUnroll; ++u) {
-        const int e = g0 + 32 * u + lane;
-        if (q[u] >= 0) {
-          const int ia = e / a.nc;
-          v[u][0] = model_value(a, i, j, l, ia, e - ia * a.nc);
-        }
-      }
+      for (int u = 0; u < UR; ++u)
+        if (q[u] >= 0) v[u][0] = model_value(a, i, j, l, g0 + u, ib);
     }
 #pragma unroll
-    for (int u = 0; u < kSumUnroll; ++u) {
-      const int q0 = __shfl_sync(0xffffffffu, q[u], 0);
-      if (__all_sync(0xffffffffu, q[u] == q0)) {
-        if (q0 != cur) {
-          flush();
-          cur = q0;
-        }
-        if (cur >= 0) {
-          cnt += 32;
+    for (int u = 0; u < UR; ++u) {
+      const bool turn = q[u] != cur;
+      const unsigned who = __ballot_sync(0xffffffffu, turn && cur >= 0);
+      if (who) flush_lanes<NB>(who, cur, run, cnt, nb, a.nbin, hs, hc, lane);
+      if (turn) {
+        cur = q[u];
+        cnt = 0;
 #pragma unroll
-          for (int b = 0; b < NB; ++b)
-            if (b < nb) run[b] += v[u][b];
-        }
-      } else {  // mixed bins: close the run, then every lane adds its own sample
-        flush();
-        cur = -1;
-        if (q[u] >= 0) {
-          atomicAdd(hc + q[u], 1u);
-#pragma unroll
-          for (int b = 0; b < NB; ++b)
-            if (b < nb) atomicAdd(hs + (size_t)b * a.nbin + q[u], v[u][b]);
-        }
+        for (int b = 0; b < NB; ++b) run[b] = 0.0;
       }
+      ++cnt;
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+        if (b < nb) run[b] += v[u][b];  // a dropped sample's sum is never flushed
     }
   }
-  flush();
+  const unsigned who = __ballot_sync(0xffffffffu, cur >= 0);
+  flush_lanes<NB>(who, cur, run, cnt, nb, a.nbin, hs, hc, lane);
   __syncthreads();
   for (int q = threadIdx.x; q < a.nbin; q += blockDim.x) {
     const unsigned c = hc[q];
@@ -245,133 +253,166 @@ __global__ void __launch_bounds__(kThreads) k_mono_sum(const MonoArgs a,
   }
 }
 
+// Rows and units of the column-walking kernels over nrows rows: as many row
+// ranges per plane as fill the chip about three times over with 32 warps per
+// SM, at least 32 rows each (a range's end flushes every lane).
+static void mono_split(MonoArgs &a, int npl, int nrows, int &gx) {
+  const int ncw = (a.nc + 31) / 32;
+  const long long units = (long long)npl * ncw;
+  const int want = (int)std::min<long long>(std::max(1, nrows / 32), (3LL * 152 * 32 + units - 1) / units);
+  a.chunk = (nrows + want - 1) / want;
+  const int nrc = (nrows + a.chunk - 1) / a.chunk;
+  gx = (ncw * nrc + kThreads / 32 - 1) / (kThreads / 32);
+}
+
+// 1 / sqrt(s) in FP64 for s in FP32's normal range: an FP32 seed (relative error
+// below 2^-19: the 20 leading mantissa bits of s, then rsqrtf) and one third-order
+// step, y (1 + e / 2 + 3 e^2 / 8) with e = 1 - s y^2, whose error 5 e^3 / 16 is below
+// 2^-55.  Five FP64 operations, against a square root and a division.
+__device__ __forceinline__ double rsqrt64(double s) {
+  const uint32_t h = (uint32_t)__double2hiint(s);
+  const uint32_t f = __float_as_uint(rsqrtf(__uint_as_float((h - (896u << 20)) << 3)));
+  const double y = __hiloint2double((int)((f >> 3) + (896u << 20)), (int)(f << 29));
+  const double e = __fma_rn(-__dmul_rn(s, y), y, 1.0);
+  return __fma_rn(__dmul_rn(y, e), __fma_rn(0.375, e, 0.5), y);
+}
+
 // m = 0 multipoles (Eq. bs_lm): per bin the sums of (2l+1) P_l(mu_1) B over the
 // paired samples, l = 0..LMAX, with mu_1 = k_par / k of the largest side (the
-// first of sides 1, 2, 3 on ties) and P_l by Bonnet's recursion, in FP64 with
-// the same operation order as the oracle.  Bins come from the plan's table.
-// Layout as k_mono_sum: warps walk 32 consecutive samples; lane-private
-// running sums while the warp's bin is unchanged.
+// first of sides 1, 2, 3 on ties; sides as the oracle rounds them).  Bins come
+// from the plan's table; the walk is k_mono_sum's.
+//
+// FP64 arithmetic bounds the kernel: one warp-wide FP64 instruction takes about
+// 18 cycles of an SM (0.5e12 a second over the part), so everything else hides
+// behind it, and the time is the count of FP64 instructions.
+//  * The row's side S1 and k_par, uniform over the warp, are computed for 32 rows
+//    at a time, one row per lane, and handed out by shuffles.
+//  * The largest side is picked on the bit patterns (positive doubles order as
+//    integers): comparisons run on the FP64 pipe too.
+//  * mu_1 by rsqrt64; the weights 1, x, (15 x^2 - 5)/2, ... as polynomials
+//    (l = 1 is multiplied by its factor 3 once per bin, at the end).
+//  * Where k_par is antisymmetric about the zero delay (a.mirror; decided on the
+//    host), the sample at (-a, -b) has the same bin and the opposite mu_1: its even
+//    multipoles take B(a, b) + B(-a, -b), its odd ones the difference, with one
+//    set of weights for the two.  11 FP64 instructions a sample, 20 unpaired.
+// 216 planes of 768^2, l <= 4: 3.1 ms; 22.4 ms before (about 90 FP64 instructions
+// a sample, and mixed groups through shared-memory FP64 atomics).
 constexpr int kMaxL = 4;
 
 template <int NB, int LMAX>
 __global__ void __launch_bounds__(kThreads) k_mono_multipole(const MonoArgs a,
                                                              const int16_t *__restrict__ bins,
                                                              int skip0) {
+  constexpr int NL = LMAX + 1, UR = NB == 1 ? 4 : 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double *hs = reinterpret_cast<double *>(smem_raw);  // [nbatch][LMAX + 1][nbin]
-  unsigned *hc = reinterpret_cast<unsigned *>(hs + (size_t)a.nbatch * (LMAX + 1) * a.nbin);
+  unsigned *hc = reinterpret_cast<unsigned *>(hs + (size_t)a.nbatch * NL * a.nbin);
   const int p = blockIdx.y;
-  for (int q = threadIdx.x; q < a.nbatch * (LMAX + 1) * a.nbin; q += blockDim.x) hs[q] = 0.0;
+  for (int q = threadIdx.x; q < a.nbatch * NL * a.nbin; q += blockDim.x) hs[q] = 0.0;
   for (int q = threadIdx.x; q < a.nbin; q += blockDim.x) hc[q] = 0u;
   __syncthreads();
   const int i = a.rings[3 * p], j = a.rings[3 * p + 1], l = a.rings[3 * p + 2];
   const double pi2 = __dmul_rn(a.kperp64[i], a.kperp64[i]),
                pj2 = __dmul_rn(a.kperp64[j], a.kperp64[j]),
                pl2 = __dmul_rn(a.kperp64[l], a.kperp64[l]);
-  const int n = a.nc * a.nc;
-  const int c0 = blockIdx.x * a.chunk, c1 = min(n, c0 + a.chunk);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kThreads / 32;
-  const int per = ((c1 - c0 + nw - 1) / nw + 31) / 32 * 32;
-  const int w0 = min(c1, c0 + warp * per), w1 = min(c1, w0 + per);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int unit = blockIdx.x * (kThreads / 32) + warp, ncw = (a.nc + 31) / 32;
+  const int ib = (unit % ncw) * 32 + lane;
+  // rows skip0 .. nc - 1, or with pairing skip0 .. nc / 2 (the zero-delay row unpaired)
+  const int h = a.nc / 2, rend = a.mirror ? h + 1 : a.nc;
+  const int ia0 = min(rend, skip0 + (unit / ncw) * a.chunk), ia1 = min(rend, ia0 + a.chunk);
+  const bool on = ib >= skip0 && ib < a.nc;
+  const double zb = on ? a.kpar64[ib] : 0.0;
+  const double s2 = __dadd_rn(pj2, __dmul_rn(zb, zb));
+  const int back = a.nc - 1 + skip0;  // index a pairs with back - a
+  const long long n = (long long)a.nc * a.nc;
   const int16_t *bp = bins + (long long)p * n;
   const double *vb = a.b3d + (long long)a.b0 * a.bstride + (long long)p * n;
   int cur = -1;
   unsigned cnt = 0;
-  double run[NB][LMAX + 1];
+  double run[NB * NL];
 #pragma unroll
-  for (int b = 0; b < NB; ++b)
+  for (int k = 0; k < NB * NL; ++k) run[k] = 0.0;
+  for (int t0 = ia0; t0 < ia1; t0 += 32) {
+    const double zr = a.kpar64[min(t0 + lane, a.nc - 1)];
+    const double s1r = __dadd_rn(pi2, __dmul_rn(zr, zr));
+    const int t1 = min(ia1, t0 + 32);
+    for (int g0 = t0; g0 < t1; g0 += UR) {
+      int q[UR];
+      double v[UR][NB], w[UR][NB];
 #pragma unroll
-    for (int q = 0; q <= LMAX; ++q) run[b][q] = 0.0;
-  auto flush = [&]() {
-    if (cur >= 0) {
+      for (int u = 0; u < UR; ++u) {
+        const int ia = g0 + u;
+        const bool live = on && ia < t1, pair = live && a.mirror && ia < h;
+        const long long e = (long long)ia * a.nc + ib;
+        const long long m = (long long)(back - ia) * a.nc + (back - ib);
+        q[u] = live ? (int)bp[e] : -1;
+        if (q[u] >= 0 && !BS_CHK(q[u], a.nbin, 42)) q[u] = -1;
 #pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        if (b >= a.nbatch) break;
-#pragma unroll
-        for (int q = 0; q <= LMAX; ++q) {
-          double x = run[b][q];
-          for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-          if (lane == 0) atomicAdd(hs + ((size_t)b * (LMAX + 1) + q) * a.nbin + cur, x);
+        for (int b = 0; b < NB; ++b) {
+          v[u][b] = (b < a.nbatch && live) ? __ldg(vb + (long long)b * a.bstride + e) : 0.0;
+          w[u][b] = (b < a.nbatch && pair) ? __ldg(vb + (long long)b * a.bstride + m) : 0.0;
         }
       }
-      if (lane == 0) atomicAdd(hc + cur, cnt);
-    }
-    cnt = 0;
 #pragma unroll
-    for (int b = 0; b < NB; ++b)
+      for (int u = 0; u < UR; ++u) {
+        const int ia = g0 + u;
+        if (ia >= t1) break;
+        const double za = __shfl_sync(0xffffffffu, zr, ia - t0);
+        const double s1 = __shfl_sync(0xffffffffu, s1r, ia - t0);
+        const bool turn = q[u] != cur;
+        const unsigned who = __ballot_sync(0xffffffffu, turn && cur >= 0);
+        if (who) flush_lanes<NB * NL>(who, cur, run, cnt, a.nbatch * NL, a.nbin, hs, hc, lane);
+        if (turn) {
+          cur = q[u];
+          cnt = 0;
 #pragma unroll
-      for (int q = 0; q <= LMAX; ++q) run[b][q] = 0.0;
-  };
-  for (int g0 = w0; g0 < w1; g0 += 32) {
-    const int e = g0 + lane;
-    int q = -1;
-    double wl[LMAX + 1];
-    if (e < w1) {
-      const int ia = e / a.nc, ib = e - ia * a.nc;
-      q = (skip0 && (ia == 0 || ib == 0)) ? -1 : (int)bp[e];
-      if (q >= 0 && !BS_CHK(q, a.nbin, 42)) q = -1;
-      if (q >= 0) {
-        const double za = a.kpar64[ia], zb = a.kpar64[ib], zc = -__dadd_rn(za, zb);
-        const double s1 = __dadd_rn(pi2, __dmul_rn(za, za)), s2 = __dadd_rn(pj2, __dmul_rn(zb, zb)),
-                     s3 = __dadd_rn(pl2, __dmul_rn(zc, zc));
-        double sm = s1, zm = za;
-        if (s2 > sm) { sm = s2; zm = zb; }
-        if (s3 > sm) { sm = s3; zm = zc; }
-        const double x = zm / sqrt(sm);
-        double pm1 = 1.0, p0 = x;
-        wl[0] = 1.0;
-        if (LMAX >= 1) wl[1] = 3.0 * x;
-#pragma unroll
-        for (int ll = 1; ll < LMAX; ++ll) {
-          const double pn = ((2 * ll + 1) * x * p0 - ll * pm1) / (ll + 1);
-          pm1 = p0;
-          p0 = pn;
-          wl[ll + 1] = (2 * ll + 3) * pn;
+          for (int k = 0; k < NB * NL; ++k) run[k] = 0.0;
         }
-      }
-    }
-    double v[NB];
+        if (!__any_sync(0xffffffffu, cur >= 0)) continue;
+        const bool pair = a.mirror && ia < h;
+        cnt += pair ? 2u : 1u;
+        double x = 0.0, x2 = 0.0;
+        if (LMAX >= 1) {
+          const double zc = -__dadd_rn(za, zb), s3 = __dadd_rn(pl2, __dmul_rn(zc, zc));
+          double sm = s1, zm = za;
+          if (__double_as_longlong(s2) > __double_as_longlong(sm)) { sm = s2; zm = zb; }
+          if (__double_as_longlong(s3) > __double_as_longlong(sm)) { sm = s3; zm = zc; }
+          x = __dmul_rn(zm, rsqrt64(sm));
+          if (LMAX >= 2) x2 = __dmul_rn(x, x);
+        }
+        const double w2 = LMAX >= 2 ? __fma_rn(7.5, x2, -2.5) : 0.0;
+        const double w3 = LMAX >= 3 ? __dmul_rn(x, __fma_rn(17.5, x2, -10.5)) : 0.0;
+        const double w4 = LMAX >= 4 ? __fma_rn(__fma_rn(39.375, x2, -33.75), x2, 3.375) : 0.0;
 #pragma unroll
-    for (int b = 0; b < NB; ++b)
-      v[b] = (b < a.nbatch && e < w1) ? __ldg(vb + (long long)b * a.bstride + e) : 0.0;
-    const int qq = __shfl_sync(0xffffffffu, q, 0);
-    if (__all_sync(0xffffffffu, q == qq)) {
-      if (qq != cur) {
-        flush();
-        cur = qq;
-      }
-      if (cur >= 0) {
-        cnt += 32;
-#pragma unroll
-        for (int b = 0; b < NB; ++b)
-#pragma unroll
-          for (int ll = 0; ll <= LMAX; ++ll)
-            if (b < a.nbatch) run[b][ll] += wl[ll] * v[b];
-      }
-    } else {
-      flush();
-      cur = -1;
-      if (q >= 0) {
-        atomicAdd(hc + q, 1u);
-#pragma unroll
-        for (int b = 0; b < NB; ++b)
-#pragma unroll
-          for (int ll = 0; ll <= LMAX; ++ll)
-            if (b < a.nbatch)
-              atomicAdd(hs + ((size_t)b * (LMAX + 1) + ll) * a.nbin + q, wl[ll] * v[b]);
+        for (int b = 0; b < NB; ++b) {
+          double ev = v[u][b], od = ev;
+          if (pair) {
+            ev = __dadd_rn(v[u][b], w[u][b]);
+            if (LMAX >= 1) od = __dsub_rn(v[u][b], w[u][b]);
+          }
+          double *r = run + b * NL;
+          r[0] += ev;
+          if constexpr (LMAX >= 1) r[1] = __fma_rn(x, od, r[1]);
+          if constexpr (LMAX >= 2) r[2] = __fma_rn(w2, ev, r[2]);
+          if constexpr (LMAX >= 3) r[3] = __fma_rn(w3, od, r[3]);
+          if constexpr (LMAX >= 4) r[4] = __fma_rn(w4, ev, r[4]);
+        }
       }
     }
   }
-  flush();
+  const unsigned who = __ballot_sync(0xffffffffu, cur >= 0);
+  flush_lanes<NB * NL>(who, cur, run, cnt, a.nbatch * NL, a.nbin, hs, hc, lane);
   __syncthreads();
   for (int q = threadIdx.x; q < a.nbin; q += blockDim.x) {
     const unsigned c = hc[q];
     if (!c) continue;
     if (a.cnt) atomicAdd(a.cnt + q, (unsigned long long)c);
     for (int b = 0; b < a.nbatch; ++b)
-      for (int ll = 0; ll <= LMAX; ++ll)
-        atomicAdd(a.sums + ((size_t)(a.b0 + b) * (LMAX + 1) + ll) * a.nbin + q,
-                  hs[((size_t)b * (LMAX + 1) + ll) * a.nbin + q]);
+      for (int ll = 0; ll <= LMAX; ++ll) {
+        const double x = hs[((size_t)b * NL + ll) * a.nbin + q];
+        atomicAdd(a.sums + ((size_t)(a.b0 + b) * NL + ll) * a.nbin + q, ll == 1 ? 3.0 * x : x);
+      }
   }
 }
 
@@ -617,11 +658,6 @@ static bs_status mono_geometry(bs_plan p, const double *kperp_host, const double
     MONO_CUDA(cudaGetLastError());
     p->mono_key.swap(key);
   }
-  // CTAs of 64 Ki samples (8 Ki per warp): few flushes, several CTAs per plane
-  const int n = nc * nc;
-  const int per_cta = 65536;
-  const int nx = std::max(1, (n + per_cta - 1) / per_cta);
-  a.chunk = ((n + nx - 1) / nx + 255) / 256 * 256;
   return BS_OK;
 }
 
@@ -690,8 +726,8 @@ bs_status bs_bs_monopole(bs_plan p, const double *b3d, const double *kperp_host,
     if (st != BS_OK) return st;
   }
   a.cnt = reinterpret_cast<unsigned long long *>(count_dev);
-  const int n = p->nc * p->nc;
-  const int gx = (n + a.chunk - 1) / a.chunk;
+  int gx = 0;
+  mono_split(a, npl, p->nc, gx);
   for (int b0 = 0; b0 < batch; b0 += per) {
     a.b0 = b0;
     a.nbatch = std::min(per, batch - b0);
@@ -759,9 +795,12 @@ bs_status bs_bs_multipoles(bs_plan p, const double *b3d, const double *kperp_hos
     if (st != BS_OK) return st;
   }
   a.cnt = reinterpret_cast<unsigned long long *>(count_dev);
-  const int n = p->nc * p->nc;
-  const int gx = (n + a.chunk - 1) / a.chunk;
   const int skip0 = p->nc % 2 == 0;  // delay index -nc/2 has no reflection on the grid
+  a.mirror = 1;
+  for (int c = skip0; c < p->nc; ++c)
+    if (kpar_host[c] != -kpar_host[p->nc - 1 + skip0 - c]) a.mirror = 0;
+  int gx = 0;
+  mono_split(a, npl, (a.mirror ? p->nc / 2 + 1 : p->nc) - skip0, gx);
   for (int b0 = 0; b0 < batch; b0 += per) {
     a.b0 = b0;
     a.nbatch = std::min(per, batch - b0);

@@ -294,6 +294,45 @@ def test_multipoles_on_estimated_bispectrum(batch, lmax, nc):
     plan.close()
 
 
+@pytest.mark.parametrize("nc,lmax,shift", [(2, 4, 0.0), (31, 4, 0.0), (32, 3, 0.0), (33, 4, 0.3),
+                                           (34, 1, 0.3), (65, 2, 0.0), (97, 0, 0.3)])
+def test_multipoles_of_planes_without_symmetry(nc, lmax, shift):
+    """Random planes (no point symmetry) with a k_par axis that is antisymmetric
+    (samples go in pairs) or shifted (one by one), at column counts around whole warps;
+    an infinite value stays in its own bin."""
+    torch = _torch()
+    import paper_2506_10526_gb300 as bs
+    edges = [1.0, 3.0, 5.0, 8.0]
+    plan = bs.Plan(16, nc, edges)
+    plan.grid_load(torch.zeros((1, nc, 16, 16), dtype=torch.complex64, device="cuda"))
+    tri, _ = plan.counts()
+    b3h = np.random.default_rng(nc).normal(size=(1, plan.n_closable, nc, nc))
+    kperp = 2 * np.pi * plan.ring_umean()
+    kpar = 9.0 * mo.kpar_axis(nc) + shift
+    k1e = np.geomspace(0.5 * kperp.min(), 1.2 * np.sqrt(kperp.max() ** 2 + 4 * kpar.max() ** 2), 8)
+    trips = _planes_trips(tri, len(edges) - 1)
+
+    def run(x):
+        s, c = plan.bs_multipoles(torch.from_numpy(x).cuda(), kperp, kpar, k1e, 3, 4, lmax=lmax)
+        m, mc = plan.bs_monopole(torch.from_numpy(x).cuda(), kperp, kpar, k1e, 3, 4)
+        return s.cpu().numpy(), c.cpu().numpy(), m.cpu().numpy(), mc.cpu().numpy()
+
+    s, c, m, mc = run(b3h)
+    _, c_o = mo.bs_multipoles(b3h, trips, kperp, kpar, k1e, 3, 4, lmax)
+    iv = mo.multipole_interval(b3h, trips, kperp, kpar, k1e, 3, 4, lmax, REL_K, REL_S)
+    _check_interval(c, s, iv, c_o, 1e-12 * np.abs(b3h).max() * 9 * np.maximum(iv["c_hi"], 1))
+    _, m_o = mo.bs_monopole(b3h, trips, kperp, kpar, k1e, 3, 4)
+    im = mo.monopole_interval(b3h, trips, kperp, kpar, k1e, 3, 4, REL_K, REL_S)
+    _check_interval(mc, m, im, m_o, 1e-12 * np.abs(b3h).max() * np.maximum(im["c_hi"], 1))
+    b3h[0, 0, nc // 2, nc - 1] = np.inf
+    si, ci, mi, _ = run(b3h)
+    np.testing.assert_array_equal(ci, c)
+    bad = ~np.isfinite(si[0, 0])
+    assert bad.sum() <= 1 and np.all(np.isfinite(si[:, :, ~bad]))
+    assert (~np.isfinite(mi)).sum() <= 1
+    plan.close()
+
+
 def test_multipoles_argument_errors():
     torch = _torch()
     import paper_2506_10526_gb300 as bs
