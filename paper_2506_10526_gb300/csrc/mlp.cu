@@ -492,7 +492,7 @@ bs_status bs_mlp_forward(bs_mlp m, const float *x_dev, int n, float *y_dev, void
   if (n == 0) return BS_OK;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (m->tc) {
-    ML_CUDA(mlp_tc_forward(m->dev, x_dev, n, nullptr, n, y_dev, nullptr, s));
+    ML_CUDA(mlp_tc_infer(m->dev, x_dev, n, y_dev, s));
     return BS_OK;
   }
   k_mlp_forward<<<(n + kRows - 1) / kRows, kRows, fwd_smem(m->dev.d, m->dev.w), s>>>(

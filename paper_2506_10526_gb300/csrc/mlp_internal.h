@@ -19,6 +19,7 @@ struct MlpDev {
 // and scratch layouts as the SIMT kernels: store rows [xn (d) | h1 (w) |
 // h2 (w) | yn], bw rows [dz1 (w) | dz2 (w) | dyn].  Width 128, d <= 64.
 bool mlp_tc_supported(int d, int w);
+cudaError_t mlp_tc_infer(const MlpDev &M, const float *x, int n, float *y, cudaStream_t s);
 cudaError_t mlp_tc_forward(const MlpDev &M, const float *x, int n, const int *idx, int nrows,
                            float *y, float *store, cudaStream_t s);
 cudaError_t mlp_tc_backward_rows(const MlpDev &M, const float *t, const int *idx, int nrows,
