@@ -73,13 +73,17 @@ struct ColEntry {
   int swapped;
 };
 
-// A (ring pair, column tile) work item of the contraction.
-struct PairTile {
-  int ri, rj;    // rings of the pair operand
-  int col_off;   // offset of this pair's column list in the column array
-  int ncol;      // columns in the pair's list
-  int col0;      // first column of this tile
-  int pad[3];
+// A column window of a ring pair in the FP32 contraction.  Its items (pair
+// rectangles x K segments x realisations) are numbered from `first` on.
+struct SimtTile {
+  int level, h;    // image level; tile form: 128 h pairs x 128 / h columns
+  int ri, rj;      // field slots of the pair operand
+  int col_off;     // offset of this pair's column list in the column array
+  int ncol;        // columns in the pair's list
+  int col0;        // first column of this window
+  int nk, kseg_len;  // K segments and their length
+  int pad;
+  long long first;
 };
 
 // Geometry shared by the field kernels.  A plan may hold fields at several
@@ -93,17 +97,20 @@ struct GridGeom {
   const int *ring_of;     // device [nslot]
 };
 
-// Contraction launch arguments.
+// FP32 contraction: the fields of one image level, and the launch arguments.
+struct SimtLevel {
+  const float *F;     // [batch][slots * nc][M2]
+  long long bstride;  // slots * nc * M2
+  int M2;
+};
+constexpr int kMaxLevels = 20;  // image sides 2^a {8, 12} up to 4096: at most 19
 struct ContractArgs {
-  const float *F;          // fields [batch][nb*nc][M*M]
-  long long fstride;       // M*M
-  long long bstride;       // nb*nc*M*M
-  int M2, nc;
+  SimtLevel lev[kMaxLevels];
+  int nc, ntile;
+  long long nitem;
   const ColEntry *cols;
-  const PairTile *ptiles;
+  const SimtTile *tiles;
   int nu1_lo, nu1_hi, nu2_lo, nu2_hi;
-  int n_r2;                // number of nu2 row blocks
-  int kseg_len, nkseg;
   const double *tnorm;     // per ring triple: 1/(A M^2 T), 0 when T == 0
   double *out_full;        // [batch][ntrip][nc][nc][nc] or null
   long long full_bstride;  // ntrip*nc^3
@@ -229,8 +236,8 @@ cudaError_t launch_effective_label(int ncell, const int8_t *label, const float *
                                   int8_t *out, cudaStream_t s);
 cudaError_t launch_counts(int nt, int nb, const int8_t *label, const int *cells, int ncells,
                           const int *trip_of, unsigned long long *T, cudaStream_t s);
-cudaError_t launch_contract_simt(const ContractArgs &a, int ntiles_row, int npt,
-                                 int batch, cudaStream_t s);
+cudaError_t launch_contract_simt(const ContractArgs &a, cudaStream_t s);
+int simt_form(int n_nu1, int n_nu2, int ncol);  // SimtTile::h of a column list
 cudaError_t launch_full_fill(double *out, long long bstride, int batch, int ntrip, int nc,
                              const int *blk, double value, cudaStream_t s);
 cudaError_t launch_full_finalize(double *out, long long bstride, int batch, int ntrip,

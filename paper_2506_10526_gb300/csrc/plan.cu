@@ -109,7 +109,7 @@ void compute_layout(bs_plan p) {
   L.T = take((size_t)p->ntrip * sizeof(unsigned long long));
   L.nnu = take(n2 * n2 * sizeof(long long));
   L.cols = take(p->max_cols * sizeof(ColEntry));
-  L.ptiles = take(p->max_ptiles * sizeof(PairTile));
+  L.ptiles = take(p->max_ptiles * sizeof(SimtTile));
   L.tctiles = take(p->max_tctiles * sizeof(TcTile));
   size_t gmax = 0;
   const bool split = p->d.precision != BS_PREC_FP32;
@@ -687,6 +687,98 @@ bs_status mabs_tc(bs_plan p, const int *blk, double *out_full, int accumulate, c
   return BS_OK;
 }
 
+// FP32 contraction of one channel block: one launch over every image side.
+static bs_status mabs_simt(bs_plan p, const int *blk, double *out_full, int accumulate,
+                           cudaStream_t s) {
+  const WsLayout &L = p->L;
+  const int nb = p->nb, nc = p->nc;
+  const int w1 = blk[1] - blk[0], w2 = blk[3] - blk[2];
+  ContractArgs a{};
+  p->h_cols.clear();
+  p->h_ptiles.clear();
+  std::vector<std::pair<double, SimtTile>> work;  // pixels of one item, entry
+  if (w1 <= 0 || w2 <= 0) return BS_OK;
+  for (int li = 0; li < (int)p->levels.size(); ++li) {
+    const Level &lv = p->levels[li];
+    const int M2 = lv.M * lv.M;
+    a.lev[li] = SimtLevel{p->at<float>(lv.offF), (long long)lv.nslot * nc * M2, M2};
+    if (lv.nslot == 0) continue;
+    // column lists over (l, nu3) with T(i,j,l) > 0 at this side and nu3 valid
+    long long windows = 0;
+    const size_t w0 = work.size();
+    for (int i = 0; i < nb; ++i)
+      for (int j = i; j < nb; ++j) {
+        const int off = (int)p->h_cols.size();
+        for (int l = j; l < nb; ++l) {
+          const int t = p->trip_of[((size_t)i * nb + j) * nb + l];
+          if (p->T[t] <= 0 || p->lev_of_trip[t] != li) continue;
+          for (int n3 = blk[4]; n3 < blk[5]; ++n3)
+            if (p->valid[n3]) p->h_cols.push_back(ColEntry{lv.slot_of[l] * nc + n3, t, n3, 0});
+        }
+        const int ncol = (int)p->h_cols.size() - off;
+        if (ncol == 0) continue;
+        windows += (ncol + 127) / 128;
+        const int h = simt_form(w1, w2, ncol);
+        for (int c0 = 0; c0 < ncol; c0 += 128 / h)
+          work.push_back({0.0, SimtTile{li, h, lv.slot_of[i], lv.slot_of[j], off, ncol, c0, 1, 0, 0, 0}});
+      }
+    if (windows > 65535) return fail(p, BS_ERR_UNSUPPORTED, "too many column tiles in one block");
+    // split K until the side's tiles cover several waves of 152 SMs.  The count is
+    // that of 128 x 128 tiles whatever the form, so that the segments (whose FP32
+    // partial sums meet in FP64) do not depend on it
+    const long long ctas = (long long)((w1 + 15) / 16) * ((w2 + 7) / 8) * windows * p->batch;
+    int nk = 1;
+    const int nchunks = M2 / 16;
+    while (ctas * nk < 4 * 152 && nk * 2 <= nchunks / 16 && nk < 64) nk *= 2;
+    while ((long long)nk * p->batch > 65535) nk /= 2;
+    for (size_t q = w0; q < work.size(); ++q) {
+      work[q].second.nk = nk;
+      work[q].second.kseg_len = ((nchunks + nk - 1) / nk) * 16;
+      work[q].first = (double)work[q].second.kseg_len;
+    }
+  }
+  if (work.empty()) return BS_OK;
+  std::stable_sort(work.begin(), work.end(),
+                   [](const std::pair<double, SimtTile> &x, const std::pair<double, SimtTile> &y) {
+                     return x.first > y.first;
+                   });
+  for (auto &w : work) {
+    SimtTile &t = w.second;
+    t.first = a.nitem;
+    a.nitem += (long long)((w1 + 15) / 16) * ((w2 + 8 * t.h - 1) / (8 * t.h)) * t.nk * p->batch;
+    p->h_ptiles.push_back(t);
+  }
+  if (p->h_ptiles.size() > p->max_ptiles || p->h_cols.size() > p->max_cols)
+    return fail(p, BS_ERR_STATE, "FP32 work list exceeds the plan's capacity");
+  const StagedUpload up[2] = {
+      {p->at<ColEntry>(L.cols), p->h_cols.data(), p->h_cols.size() * sizeof(ColEntry)},
+      {p->at<SimtTile>(L.ptiles), p->h_ptiles.data(), p->h_ptiles.size() * sizeof(SimtTile)}};
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+  if (cap == cudaStreamCaptureStatusActive) {  // no event waits inside a capture
+    for (const StagedUpload &u : up)
+      BS_CUDA(cudaMemcpyAsync(u.dst, u.src, u.bytes, cudaMemcpyHostToDevice, s));
+  } else {
+    bs_status st = upload_staged(p, s, up, 2);
+    if (st != BS_OK) return st;
+  }
+  a.ntile = (int)p->h_ptiles.size();
+  a.nc = nc;
+  a.cols = p->at<ColEntry>(L.cols);
+  a.tiles = p->at<SimtTile>(L.ptiles);
+  a.nu1_lo = blk[0];
+  a.nu1_hi = blk[1];
+  a.nu2_lo = blk[2];
+  a.nu2_hi = blk[3];
+  a.tnorm = p->at<double>(L.tnorm);
+  a.out_full = out_full;
+  a.full_bstride = (long long)p->ntrip * nc * nc * nc;
+  a.dsum = accumulate ? p->at<double>(L.dsum) : nullptr;
+  a.dsum_bstride = (long long)p->ntrip * (2 * nc - 1) * (2 * nc - 1);
+  BS_CUDA(launch_contract_simt(a, s));
+  return BS_OK;
+}
+
 // Scratch of a general plan for the four real components of an output (grown on
 // demand with cudaMalloc, freed with the plan).
 bs_status general_scratch(bs_plan p, double **buf, size_t *cap, size_t n) {
@@ -956,7 +1048,8 @@ bs_status bs_plan_create(const bs_plan_desc *desc, bs_plan *out) {
   p->nnu.assign((size_t)(2 * p->nc - 1) * (2 * p->nc - 1), 0);
   const int npairs = p->nb * (p->nb + 1) / 2;
   p->max_cols = (size_t)npairs * p->nb * p->nc;
-  p->max_ptiles = (size_t)npairs * ((size_t)p->nb * p->nc / 128 + 1);
+  // FP32 column windows: 32 columns at the narrowest, one part-filled window per level
+  p->max_ptiles = (size_t)npairs * ((size_t)p->nb * p->nc / 32 + p->levels.size());
   // tensor-core tiles: pair rectangles (32 x 16) x 256-entry column windows (runs padded to 8)
   cudaDeviceGetAttribute(&p->nsm, cudaDevAttrMultiProcessorCount, dev);
   if (p->d.precision != BS_PREC_FP32) {
@@ -1153,63 +1246,8 @@ bs_status bs_mabs(bs_plan p, const int32_t *block, double *out_full, int accumul
     st = mabs_tc(p, blk, out_full, accumulate, s);
     if (st != BS_OK) return st;
   } else {
-    // one launch per image side: work list of ring pairs (i <= j) x column tiles over
-    // (l, nu3) with T(i,j,l) > 0 at this side and nu3 valid; rings are this level's slots
-    const int nb = p->nb;
-    for (int li = 0; li < (int)p->levels.size(); ++li) {
-      const Level &lv = p->levels[li];
-      if (lv.nslot == 0) continue;
-      p->h_cols.clear();
-      p->h_ptiles.clear();
-      for (int i = 0; i < nb; ++i)
-        for (int j = i; j < nb; ++j) {
-          const int off = (int)p->h_cols.size();
-          for (int l = j; l < nb; ++l) {
-            const int t = p->trip_of[((size_t)i * nb + j) * nb + l];
-            if (p->T[t] <= 0 || p->lev_of_trip[t] != li) continue;
-            for (int n3 = blk[4]; n3 < blk[5]; ++n3)
-              if (p->valid[n3]) p->h_cols.push_back(ColEntry{lv.slot_of[l] * nc + n3, t, n3, 0});
-          }
-          const int ncol = (int)p->h_cols.size() - off;
-          for (int c0 = 0; c0 < ncol; c0 += 128)
-            p->h_ptiles.push_back(PairTile{lv.slot_of[i], lv.slot_of[j], off, ncol, c0, {0, 0, 0}});
-        }
-      const int n_r1 = (blk[1] - blk[0] + 15) / 16, n_r2 = (blk[3] - blk[2] + 7) / 8;
-      const int npt = (int)p->h_ptiles.size();
-      if (npt == 0 || n_r1 == 0 || n_r2 == 0) continue;
-      if (npt > 65535) return fail(p, BS_ERR_UNSUPPORTED, "too many column tiles in one block");
-      BS_CUDA(cudaMemcpyAsync(p->at<ColEntry>(L.cols), p->h_cols.data(),
-                              p->h_cols.size() * sizeof(ColEntry), cudaMemcpyHostToDevice, s));
-      BS_CUDA(cudaMemcpyAsync(p->at<PairTile>(L.ptiles), p->h_ptiles.data(),
-                              p->h_ptiles.size() * sizeof(PairTile), cudaMemcpyHostToDevice, s));
-      ContractArgs a{};
-      a.F = p->at<float>(lv.offF);
-      a.fstride = (long long)lv.M * lv.M;
-      a.bstride = (long long)lv.nslot * nc * lv.M * lv.M;
-      a.M2 = lv.M * lv.M;
-      a.nc = nc;
-      a.cols = p->at<ColEntry>(L.cols);
-      a.ptiles = p->at<PairTile>(L.ptiles);
-      a.nu1_lo = blk[0];
-      a.nu1_hi = blk[1];
-      a.nu2_lo = blk[2];
-      a.nu2_hi = blk[3];
-      a.n_r2 = n_r2;
-      // split K until the launch covers several waves of 152 SMs
-      const long long ctas = (long long)n_r1 * n_r2 * npt * p->batch;
-      int nk = 1;
-      const int nchunks = a.M2 / 16;
-      while (ctas * nk < 4 * 152 && nk * 2 <= nchunks / 16 && nk < 64) nk *= 2;
-      while ((long long)nk * p->batch > 65535) nk /= 2;
-      a.nkseg = nk;
-      a.kseg_len = ((nchunks + nk - 1) / nk) * 16;
-      a.tnorm = p->at<double>(L.tnorm);
-      a.out_full = out_full;
-      a.full_bstride = full_bstride;
-      a.dsum = accumulate ? p->at<double>(L.dsum) : nullptr;
-      a.dsum_bstride = (long long)p->ntrip * (2 * nc - 1) * (2 * nc - 1);
-      BS_CUDA(launch_contract_simt(a, n_r1 * n_r2, npt, p->batch, s));
-    }
+    st = mabs_simt(p, blk, out_full, accumulate, s);
+    if (st != BS_OK) return st;
   }
   if (out_full)
     BS_CUDA(launch_full_finalize(out_full, full_bstride, p->batch, p->ntrip, nc, blk,

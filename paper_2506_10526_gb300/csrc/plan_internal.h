@@ -126,7 +126,7 @@ struct bs_plan_s {
   bool ws_owned = false;
   size_t max_cols = 0, max_ptiles = 0, max_tctiles = 0;
   std::vector<ColEntry> h_cols;
-  std::vector<PairTile> h_ptiles;
+  std::vector<SimtTile> h_ptiles;
   std::vector<TcTile> h_tctiles;
 
   bool maps_ready = false;

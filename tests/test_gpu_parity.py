@@ -422,3 +422,45 @@ def test_delay_transform_against_oracle(nc, block):
         err = np.abs(got[k] - want[k]).max() / np.abs(want[k]).max()
         assert err < TOL_FP32, (k, err)
     plan.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("block", [(0, 16, 0, 8, 0, 36), (1, 17, 3, 19, 5, 25), (0, 5, 0, 33, 2, 12),
+                                   (3, 36, 1, 18, 0, 7), (0, 36, 0, 36, 35, 36),
+                                   (7, 24, 9, 10, 0, 36)])
+def test_contraction_forms_over_ragged_blocks(block, precision):
+    """Channel blocks whose column lists and pair rectangles fill the contractions'
+    tiles to different parts (the FP32 tiles of 128, 256 and 512 pairs, the
+    tensor-core tile for short lists with one and two halves and windows),
+    image sides of 4.5 to 8 pixel stages: the collapse sums of the whole block
+    against the oracle, and the sums of two blocks that meet in one plane."""
+    torch = _torch()
+    import paper_2506_10526_gb300 as bs
+    nt, nc, edges = 12, 36, [1.0, 2.2, 3.5, 5.0]
+    vis = synth.sky_visibilities(nt, nc, seed=77)
+    ref, babs = _oracle(vis, edges)
+    b = block
+    rest = (b[0], b[1], b[2], b[3], 0, b[4])  # the same pairs, the nu3 below the block
+    for multires in (False, True):
+        plan = bs.Plan(nt, nc, edges, precision=precision, multires=multires)
+        plan.grid_load(torch.from_numpy(vis[None].astype(np.complex64)).cuda())
+        for blocks in ([b], [b, rest]):
+            plan.delta_reset()
+            for q in blocks:
+                plan.mabs(block=q)
+            sums, nnu = plan.delta_export()
+            torch.cuda.synchronize()
+            got, sides = sums[0].cpu().numpy(), plan.trip_sides()
+            lo3 = min(q[4] for q in blocks)
+            n1, n2, n3 = np.meshgrid(np.arange(b[0], b[1]), np.arange(b[2], b[3]),
+                                     np.arange(lo3, b[5]), indexing="ij")
+            at = (n1 - n3 + nc - 1, n2 - n3 + nc - 1)
+            for t in range(plan.ntrip):
+                want = np.zeros((2 * nc - 1, 2 * nc - 1))
+                size = np.zeros_like(want)
+                if ref["T"][t] > 0:
+                    scale = float(sides[t]) ** 2 * ref["T"][t]
+                    np.add.at(want, at, ref["B"][t].real[n1, n2, n3] * scale)
+                    np.add.at(size, at, babs[t][n1, n2, n3] * scale)
+                assert np.all(np.abs(got[t] - want) <= TOL[precision] * size)
+        plan.close()
