@@ -152,15 +152,20 @@ struct TcGroup {
   int nslot;
 };
 
+// Tensor maps per image level: hi, lo with boxes of 8, 32 and 128 field rows (0-5),
+// FP32 rows by 8 (6), hi, lo with boxes of 16 and 64 rows (7-10), FP32 rows by 16 (11).
+constexpr int kTcMaps = 12;
+
 struct TcArgs {
   const TcGroup *groups;   // device
-  const void *maps;        // device: 2 CUtensorMap (hi, lo) per group, 64-byte aligned
+  const void *maps;        // device: kTcMaps CUtensorMap per group, 64-byte aligned
   const TcTile *tiles;     // device
   int ntiles;
   int *err;                // device error word: 1 = a bounded wait gave up
   long long wait_limit_ns;
   int stall_test;          // failure injection: the MMA thread waits on a barrier nobody arrives at
-  int f16;                 // 1: split-FP16 operands (two products), 0: split BF16 (three)
+  int f16;                 // 1: split-FP16 operands, 0: split BF16
+  int small;               // 1: the kernel for short column lists (contract_tcs.cu)
 };
 
 // NVTX range over an entry point, named after it (no cost unless a profiler
@@ -237,6 +242,11 @@ cudaError_t launch_effective_label(int ncell, const int8_t *label, const float *
 cudaError_t launch_counts(int nt, int nb, const int8_t *label, const int *cells, int ncells,
                           const int *trip_of, unsigned long long *T, cudaStream_t s);
 cudaError_t launch_contract_simt(const ContractArgs &a, cudaStream_t s);
+// The same contraction for short column lists (contract_tcs.cu), and the rule that
+// chooses it: whether it is the faster kernel for these tiles (and can run them).
+cudaError_t launch_contract_tcs(const TcArgs &a, int nsm, cudaStream_t s);
+bool tcs_wins(const TcTile *tiles, size_t ntiles, const TcGroup *groups, const ColEntry *cols,
+              bool fixed_order);
 int simt_form(int n_nu1, int n_nu2, int ncol);  // SimtTile::h of a column list
 cudaError_t launch_full_fill(double *out, long long bstride, int batch, int ntrip, int nc,
                              const int *blk, double value, cudaStream_t s);

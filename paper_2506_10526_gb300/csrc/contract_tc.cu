@@ -100,8 +100,7 @@ constexpr int RAW_ROWS = 16 + P2;         // 16 rows of F_i (8 per half), 16 of 
 constexpr int RAW_BYTES = RAW_ROWS * KC * 4;  // 4 KB: 128-byte rows, 128B swizzle
 constexpr int RAW_BOX_BYTES = 8 * KC * 4;     // one TMA box: 8 rows
 constexpr int MAX_SEG = 16;
-// tensor maps per level: hi/lo with boxes of 8, 32 and 128 field rows, FP32 rows
-constexpr int NMAPS = 7;
+constexpr int NMAPS = kTcMaps;  // tensor maps per level: 0-5 hi/lo boxes, 6 FP32 rows
 // a_full, a_empty, pfull per field stage; b_full, b_empty per pair stage; raw_full,
 // raw_empty per row stage; acc_full, acc_empty, stall
 constexpr int NBAR = 3 * ASTAGES + 2 * STAGES + 2 * RSTAGES + 3;
@@ -748,6 +747,7 @@ int tc_smem_bytes(int f16) { return f16 ? Lay<true>::SMEM_BYTES : Lay<false>::SM
 
 cudaError_t launch_contract_tc(const TcArgs &a, int nsm, cudaStream_t s) {
   if (a.ntiles == 0) return cudaSuccess;
+  if (a.small) return launch_contract_tcs(a, nsm, s);
   return a.f16 ? launch_tc<true>(a, nsm, s) : launch_tc<false>(a, nsm, s);
 }
 

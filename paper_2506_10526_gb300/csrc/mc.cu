@@ -90,6 +90,7 @@ struct bs_mc_s {
   unsigned char *maps = nullptr;
   int *errw = nullptr;
   int ntiles = 0, nsm = 152;
+  int small = 0;                // 1: the contraction kernel for short column lists
   int f16 = 0;                  // 1: split-FP16 groups (two-product contraction)
   int min_tiles_factor = 2;     // autotuner knob: K splitting target (tiles per SM)
   int tile_order = 0;           // autotuner knob: 0 longest K first, 1 ring-pair order
@@ -206,6 +207,9 @@ bs_status mc_prepare(bs_mc m, cudaStream_t s) {
   MC_CUDA(cudaMemcpy(m->maps, maps.data(), maps.size(), cudaMemcpyHostToDevice));
   MC_CUDA(cudaMemset(m->errw, 0, sizeof(int)));
   m->ntiles = (int)tiles.size();
+  // an ensemble restored from a checkpoint goes on with the same sums: the kernel with
+  // the fixed order only where the other one's is fixed too
+  m->small = tcs_wins(tiles.data(), tiles.size(), tgs.data(), cols.data(), true) ? 1 : 0;
   m->prepared = true;
   return BS_OK;
 }
@@ -229,6 +233,7 @@ bs_status mc_enqueue(bs_mc m, cudaStream_t s) {
   a.wait_limit_ns = 2000000000LL;
   a.stall_test = 0;
   a.f16 = m->f16;
+  a.small = m->small;
   MC_CUDA(launch_contract_tc(a, m->nsm, s));
   for (Group &gr : m->groups) {
     bs_plan p = gr.plan;

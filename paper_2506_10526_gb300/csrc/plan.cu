@@ -139,7 +139,7 @@ void compute_layout(bs_plan p) {
                  (size_t)p->nc * p->nc * sizeof(double) + (size_t)p->nc);
   L.herm = take(2 * sizeof(float));
   L.err = take(sizeof(int));
-  L.maps = take(7 * p->levels.size() * sizeof(CUtensorMap));
+  L.maps = take(kTcMaps * p->levels.size() * sizeof(CUtensorMap));
   L.tcgroup = take(p->levels.size() * sizeof(TcGroup));
   L.mlptab = take(((size_t)p->ntrip * 4 + 36) * sizeof(float));
   L.ztrips = take((size_t)p->ntrip * sizeof(int));
@@ -234,9 +234,9 @@ bs_status check_device_error(bs_plan p, cudaStream_t s) {
 
 // Tensor maps over the field arrays of each level: rows = batch * nf fields,
 // inner dimension = M^2 pixels.  hi / lo (BF16, or FP16 in split-FP16
-// plans): boxes of 32 pixels x 8, 32 or 128 fields, 64-byte swizzle (the MMA operand layout; the contraction loads
+// plans): boxes of 32 pixels x 8, 16, 32, 64 or 128 fields, 64-byte swizzle (the MMA operand layout; the contraction loads
 // runs of consecutive fields with the larger boxes).  FP32 F: boxes of 32
-// pixels x 8 fields, 128-byte swizzle (the pair producers' input rows).
+// pixels x 8 or 16 fields, 128-byte swizzle (the pair producers' input rows).
 bs_status ensure_tensor_maps(bs_plan p, cudaStream_t s) {
   if (p->maps_ready) return BS_OK;
   void *fn = nullptr;
@@ -253,13 +253,14 @@ bs_status ensure_tensor_maps(bs_plan p, cudaStream_t s) {
     const cuuint64_t M2 = (cuuint64_t)lv.M * lv.M;
     cuuint64_t dims[2] = {M2, (cuuint64_t)p->batch * std::max(1, lv.nslot) * p->nc};
     cuuint32_t estr[2] = {1, 1};
-    for (int w = 0; w < 7; ++w) {
-      const bool f32 = (w == 6);
-      static const cuuint32_t rows[7] = {8, 8, 32, 32, 128, 128, 8};
+    for (int w = 0; w < kTcMaps; ++w) {
+      const bool f32 = w == 6 || w == 11;
+      const bool lo = w < 6 ? w % 2 == 1 : w % 2 == 0;
+      static const cuuint32_t rows[kTcMaps] = {8, 8, 32, 32, 128, 128, 8, 16, 16, 64, 64, 16};
       cuuint64_t strides[1] = {M2 * (f32 ? 4 : 2)};
       cuuint32_t box[2] = {32, rows[w]};
       void *base = f32 ? (void *)p->at<float>(lv.offF)
-                       : (void *)p->at<uint16_t>(w % 2 == 0 ? lv.offFhi : lv.offFlo);
+                       : (void *)p->at<uint16_t>(lo ? lv.offFlo : lv.offFhi);
       const CUtensorMapDataType half_t = p->d.precision == BS_PREC_SPLIT_FP16
                                              ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                              : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
@@ -660,6 +661,10 @@ static bs_status mabs_tc_launch(bs_plan p, const int *blk, double *out_full, int
   const char *inj = std::getenv("BS_INJECT_MMA_STALL");
   a.stall_test = (inj && inj[0] == '1') ? 1 : 0;
   a.f16 = p->d.precision == BS_PREC_SPLIT_FP16 ? 1 : 0;
+  a.small = tcs_wins(p->h_tctiles.data(), p->h_tctiles.size(), p->h_groups.data(),
+                     p->h_cols.data(), false)
+                ? 1
+                : 0;
   if (a.stall_test) a.wait_limit_ns = 50000000LL;
   BS_CUDA(launch_contract_tc(a, p->nsm, s));
   return BS_OK;

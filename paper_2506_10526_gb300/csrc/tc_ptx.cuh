@@ -1,5 +1,5 @@
-// tcgen05, TMA and mbarrier instruction forms and the operand splits of the
-// tensor-core contraction (contract_tc.cu).
+// tcgen05, TMA and mbarrier instruction forms and the operand splits shared by
+// the two tensor-core contraction kernels (contract_tc.cu, contract_tcs.cu).
 #pragma once
 
 #include <cuda.h>
@@ -110,6 +110,57 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
       "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
+// The copies of a list of 16 groups of 8 field rows: lane g < 16 has group g's first
+// row (`live`: a group of the list).  Runs of consecutive rows become one box of 16,
+// 32, 64 or 128 rows.  Fills list[0..n) with (row, byte offset of the group in a
+// 64-byte-row operand, address of the map) and returns n; mg: the level's hi maps, or
+// one on, its lo maps.  Called by a whole warp.
+__device__ __forceinline__ int box_list(const CUtensorMap *mg, int row, bool live, int4 *list,
+                                        int lane) {
+  int box = lane < 16 && live ? 1 : 0;  // rows / 8; 0: covered by an earlier box
+#pragma unroll
+  for (int n = 2; n <= 16; n *= 2) {
+    const int pbox = __shfl_down_sync(0xffffffffu, box, n / 2);
+    const int prow = __shfl_down_sync(0xffffffffu, row, n / 2);
+    const int join = (lane & (n - 1)) == 0 && box == n / 2 && pbox == n / 2 && prow == row + 4 * n;
+    const int joined = __shfl_up_sync(0xffffffffu, join, n / 2);
+    if (join) box = n;
+    if ((lane & (n - 1)) == n / 2 && joined) box = 0;
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, box > 0);
+  if (box > 0) {
+    const uint64_t mp =
+        (uint64_t)(mg + (box == 1 ? 0 : box == 2 ? 7 : box == 4 ? 2 : box == 8 ? 9 : 4));
+    list[__popc(m & ((1u << lane) - 1))] =
+        make_int4(row, lane * 8 * 64, (int)(uint32_t)mp, (int)(uint32_t)(mp >> 32));
+  }
+  __syncwarp();
+  return __popc(m);
+}
+__device__ __forceinline__ const CUtensorMap *box_map(const int4 &x) {
+  return reinterpret_cast<const CUtensorMap *>((uint64_t)(uint32_t)x.z | ((uint64_t)(uint32_t)x.w << 32));
+}
+// The first four boxes of a list in registers (a read of the list on every stage lies
+// on the issuing thread's path), the others from shared memory.
+struct Boxes {
+  int4 b[4];
+  int n;
+  const int4 *list;
+  __device__ __forceinline__ Boxes(const int4 *l, int nbox) : n(nbox), list(l) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = q < nbox ? l[q] : make_int4(0, 0, 0, 0);
+  }
+  // the copies of one stage (pixels kc..) to dst
+  __device__ __forceinline__ void load(uint32_t dst, int kc, uint32_t bar) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q < n) tma_load_2d(dst + b[q].y, box_map(b[q]), kc, b[q].x, bar);
+    for (int q = 4; q < n; ++q) {
+      const int4 x = list[q];
+      tma_load_2d(dst + x.y, box_map(x), kc, x.x, bar);
+    }
+  }
+};
 __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
