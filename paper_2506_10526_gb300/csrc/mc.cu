@@ -30,24 +30,75 @@ using namespace bsi;
 
 namespace {
 
-// Welford update over the batch dimension: x[b][n] -> (count, mean, M2)[n].
+// The statistics of a bin over realisations: count, mean and the sum of squared
+// deviations, NaN values skipped.  CH values at a time: their own mean and sum of
+// squared deviations (3 FP64 operations a value), merged into the running ones by
+// the pairwise update of Chan, Golub & LeVeque (one division per CH values).  FP64
+// issue bounds the kernel, not HBM; Welford's update, which CH = 1 keeps for fewer
+// than four realisations, takes a division for every value (256 realisations of the
+// 64^2 x 16 channel grid: 0.63 ms per call of the 3D bispectrum and the collapse).
+__device__ __forceinline__ bool is_nan_bits(double v) {
+  const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  return h > 0x7ff00000u || (h == 0x7ff00000u && __double2loint(v) != 0);
+}
+
+template <int CH>
 __global__ void k_welford(const double *__restrict__ x, int batch, long long n, double *cnt,
                           double *mean, double *m2) {
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
        j += (long long)gridDim.x * blockDim.x) {
     double c = cnt[j], mu = mean[j], s = m2[j];
-    for (int b = 0; b < batch; ++b) {
-      const double v = x[(long long)b * n + j];
-      if (v != v) continue;
-      c += 1.0;
-      const double d = v - mu;
-      mu += d / c;
-      s += d * (v - mu);
+    if constexpr (CH == 1) {
+      for (int b = 0; b < batch; ++b) {
+        const double v = x[(long long)b * n + j];
+        if (is_nan_bits(v)) continue;
+        c += 1.0;
+        const double d = v - mu;
+        mu += d / c;
+        s += d * (v - mu);
+      }
+    } else {
+      for (int b0 = 0; b0 < batch; b0 += CH) {
+        double v[CH], sum = 0.0, q = 0.0;
+        int k = 0;
+#pragma unroll
+        for (int u = 0; u < CH; ++u)
+          v[u] = b0 + u < batch ? x[(long long)(b0 + u) * n + j]
+                                : __longlong_as_double(0x7ff8000000000000LL);
+#pragma unroll
+        for (int u = 0; u < CH; ++u)
+          if (!is_nan_bits(v[u])) {
+            sum += v[u];
+            ++k;
+          }
+        if (k == 0) continue;
+        const double kd = (double)k, mb = sum / kd;
+#pragma unroll
+        for (int u = 0; u < CH; ++u)
+          if (!is_nan_bits(v[u])) {
+            const double d = v[u] - mb;
+            q = fma(d, d, q);
+          }
+        const double tot = c + kd, d = mb - mu, r = kd / tot;
+        s += fma(d * d, c * r, q);
+        mu = fma(d, r, mu);
+        c = tot;
+      }
     }
     cnt[j] = c;
     mean[j] = mu;
     m2[j] = s;
   }
+}
+
+void launch_welford(const double *x, int batch, long long n, double *st, cudaStream_t s) {
+  const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
+  if (batch >= 16)
+    k_welford<16><<<blocks, 256, 0, s>>>(x, batch, n, st, st + n, st + 2 * n);
+  else if (batch >= 4)
+    k_welford<4><<<blocks, 256, 0, s>>>(x, batch, n, st, st + n, st + 2 * n);
+  else
+    k_welford<1><<<blocks, 256, 0, s>>>(x, batch, n, st, st + n, st + 2 * n);
 }
 
 __global__ void k_welford_final(long long n, const double *cnt, const double *mean,
@@ -247,13 +298,9 @@ bs_status mc_enqueue(bs_mc m, cudaStream_t s) {
     MC_CUDA(launch_bs3d(p->at<double>(L.dsum), p->at<long long>(L.nnu), p->at<double>(L.tnorm),
                         p->at<float2>(L.tmp3d), gr.bout, p->batch, p->ntrip, p->nc,
                         p->at<float2>(L.twN), p->radN, p->scale3d, nullptr, 0, s));
-    const int blocks = (int)std::min<long long>((gr.nd + 255) / 256, 4096);
-    k_welford<<<blocks, 256, 0, s>>>(gr.dout, p->batch, gr.nd, gr.stats, gr.stats + gr.nd,
-                                     gr.stats + 2 * gr.nd);
+    launch_welford(gr.dout, p->batch, gr.nd, gr.stats, s);
     MC_CUDA(cudaGetLastError());
-    double *s3 = gr.stats + 3 * gr.nd;
-    const int blocks3 = (int)std::min<long long>((gr.nb3 + 255) / 256, 4096);
-    k_welford<<<blocks3, 256, 0, s>>>(gr.bout, p->batch, gr.nb3, s3, s3 + gr.nb3, s3 + 2 * gr.nb3);
+    launch_welford(gr.bout, p->batch, gr.nb3, gr.stats + 3 * gr.nd, s);
     MC_CUDA(cudaGetLastError());
   }
   return BS_OK;
