@@ -67,18 +67,28 @@ namespace {
 constexpr double kU = 1.0 / 16777216.0;  // 2^-24
 constexpr int kNormThreads = 512;
 
-// Per-field norms of one level's FP32 fields [nfield][m2]: out[3 f + 0..2] =
-// max |F|, ||F||_2, ||F||_3.  One CTA per field: pass 1 finds the maximum,
-// pass 2 sums (|F| / 2^e)^2 and (|F| / 2^e)^3 with 2^e > max, so that every
-// term is below 1 (no FP32 overflow), per thread in FP32 and across the CTA
-// in FP64.
-__global__ void __launch_bounds__(kNormThreads) k_field_norms(const float *__restrict__ F,
-                                                               long long m2,
-                                                               double *__restrict__ out) {
+// The FP32 fields of every level: level q holds fields first[q] .. first[q + 1] - 1
+// of m2[q] pixels.
+struct NormLevels {
+  const float *F[kMaxLevels];
+  long long m2[kMaxLevels];
+  int first[kMaxLevels + 1];
+};
+
+// Per-field norms: out[3 f + 0..2] = max |F|, ||F||_2, ||F||_3.  One CTA per
+// field: pass 1 finds the maximum, pass 2 sums (|F| / 2^e)^2 and (|F| / 2^e)^3
+// with 2^e > max, so that every term is below 1 (no FP32 overflow), per thread in
+// FP32 and across the CTA in FP64.  All levels in one launch: a launch per level
+// left the chip to 16 channels' fields at a time.
+__global__ void __launch_bounds__(kNormThreads)
+    k_field_norms(const __grid_constant__ NormLevels L, double *__restrict__ out) {
   __shared__ float smax[kNormThreads / 32];
   __shared__ double s2s[kNormThreads / 32], s3s[kNormThreads / 32];
   __shared__ float bmax;
-  const float *f = F + (long long)blockIdx.x * m2;
+  int lv = 0;
+  while ((int)blockIdx.x >= L.first[lv + 1]) ++lv;
+  const long long m2 = L.m2[lv];
+  const float *f = L.F[lv] + (long long)(blockIdx.x - L.first[lv]) * m2;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float mx = 0.f;
   for (long long x = threadIdx.x; x < m2; x += blockDim.x) mx = fmaxf(mx, fabsf(f[x]));
@@ -128,40 +138,41 @@ struct BoundLevel {
   const double *norms;  // [batch][nslot][nc][3] of this level
   const int *slot_of;   // [nb]
   const int *kexp;      // [batch][nslot] scale exponents (split FP16), else null
-  int level, nslot, nc, ntrip;
-  int batch;            // realisations written (the caller's, or internal for mode 2)
-  int mode;             // 0 bound of S / (A M^2 T); 1 general plan: four evaluations per
-                        // realisation (t = 0, 1, -1, 2); 2 bound of each internal
-                        // evaluation's S, not normalised
+  int nslot;
   double c1;            // c_term + c_acc
   double cf;            // eps_fft
   double floor16;       // 2^-25 (2^14 + 2^7) M^2 (split FP16), else 0
 };
 
-// Largest norm k (0 max, 1 2-norm, 2 3-norm) over the channels of ring r's fields.
-__device__ double ring_max(const BoundLevel &L, int b, int r, int k) {
-  const int slot = L.slot_of[r];
-  const double *n = L.norms + ((long long)b * L.nslot + slot) * L.nc * 3;
-  double m = 0.0;
-  for (int c = 0; c < L.nc; ++c) m = fmax(m, n[3 * c + k]);
-  return m;
-}
+struct BoundArgs {
+  BoundLevel lev[kMaxLevels];
+  int nc, ntrip;
+  int batch;            // realisations written (the caller's, or internal for mode 2)
+  int mode;             // 0 bound of S / (A M^2 T); 1 general plan: four evaluations per
+                        // realisation (t = 0, 1, -1, 2); 2 bound of each internal
+                        // evaluation's S, not normalised
+};
 
 // First-order bound on |dS| of one real evaluation (internal realisation b) of
-// the ring triple with rings r.
-__device__ double trip_beta(const BoundLevel &L, int b, const int r[3]) {
-  double ninf[3], n2[3], n3[3];
+// the ring triple with rings r.  Called by a whole warp, the lanes over the
+// channels: the norms are the largest over each ring's fields.
+__device__ double trip_beta(const BoundLevel &L, int nc, int b, const int r[3]) {
+  double nm[3][3];  // [ring][max, 2-norm, 3-norm]
   for (int q = 0; q < 3; ++q) {
-    ninf[q] = ring_max(L, b, r[q], 0);
-    n2[q] = ring_max(L, b, r[q], 1);
-    n3[q] = ring_max(L, b, r[q], 2);
+    const double *n = L.norms + ((long long)b * L.nslot + L.slot_of[r[q]]) * nc * 3;
+    for (int k = 0; k < 3; ++k) nm[q][k] = 0.0;
+    for (int c = threadIdx.x & 31; c < nc; c += 32)
+      for (int k = 0; k < 3; ++k) nm[q][k] = fmax(nm[q][k], n[3 * c + k]);
+    for (int k = 0; k < 3; ++k)
+      for (int o = 16; o; o >>= 1)
+        nm[q][k] = fmax(nm[q][k], __shfl_xor_sync(0xffffffffu, nm[q][k], o));
   }
   double fft = 0.0;
   for (int q = 0; q < 3; ++q) {
     const int a = (q + 1) % 3, c = (q + 2) % 3;
-    fft += n2[q] * fmin(ninf[a] * n2[c], n2[a] * ninf[c]);
+    fft += nm[q][1] * fmin(nm[a][0] * nm[c][1], nm[a][1] * nm[c][0]);
   }
-  double beta = L.c1 * n3[0] * n3[1] * n3[2] + L.cf * fft;
+  double beta = L.c1 * nm[0][2] * nm[1][2] * nm[2][2] + L.cf * fft;
   if (L.kexp) {
     const int *k = L.kexp + (long long)b * L.nslot;
     const int ks = k[L.slot_of[r[0]]] + k[L.slot_of[r[1]]] + k[L.slot_of[r[2]]];
@@ -170,29 +181,29 @@ __device__ double trip_beta(const BoundLevel &L, int b, const int r[3]) {
   return beta;
 }
 
-// bound[b][trip] for the ring triples of one level (table: i, j, l, level).
-__global__ void k_trip_bound(BoundLevel L, const int *__restrict__ tab,
+// bound[b][trip] of every ring triple (table: i, j, l, level), a warp each.  One
+// thread each walked nine dependent rows of norms per ring triple, a launch per level:
+// 12 us each for 16 channels.
+__global__ void k_trip_bound(const __grid_constant__ BoundArgs A, const int *__restrict__ tab,
                              const double *__restrict__ tnorm, double *__restrict__ bound) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= L.batch * L.ntrip) return;
-  const int b = t / L.ntrip, trip = t - b * L.ntrip;
-  if (tab[4 * trip + 3] != L.level || !(tnorm[trip] > 0.0)) return;
+  const int t = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
+  if (t >= A.batch * A.ntrip) return;
+  const int b = t / A.ntrip, trip = t - b * A.ntrip;
+  if (tab[4 * trip + 3] < 0 || !(tnorm[trip] > 0.0)) return;
+  const BoundLevel &L = A.lev[tab[4 * trip + 3]];
   const int r[3] = {tab[4 * trip], tab[4 * trip + 1], tab[4 * trip + 2]};
-  if (L.mode == 2) {
-    bound[(long long)b * L.ntrip + trip] = 1.01 * trip_beta(L, b, r);
-    return;
-  }
   double beta;
-  if (L.mode == 0) {
-    beta = trip_beta(L, b, r);
+  if (A.mode != 1) {
+    beta = trip_beta(L, A.nc, b, r);
   } else {  // evaluations t = 0, 1, -1, 2 of realisation b are internal 4b .. 4b + 3
-    const double b0 = trip_beta(L, 4 * b, r), b1 = trip_beta(L, 4 * b + 1, r),
-                 bm = trip_beta(L, 4 * b + 2, r), b2 = trip_beta(L, 4 * b + 3, r);
+    const double b0 = trip_beta(L, A.nc, 4 * b, r), b1 = trip_beta(L, A.nc, 4 * b + 1, r),
+                 bm = trip_beta(L, A.nc, 4 * b + 2, r), b2 = trip_beta(L, A.nc, 4 * b + 3, r);
     const double re = 2.0 * b0 + 0.5 * (b1 + bm);
     const double im = (9.0 * b1 + bm + 2.0 * b2 + 6.0 * b0) / 6.0;
     beta = sqrt(re * re + im * im);
   }
-  bound[(long long)b * L.ntrip + trip] = 1.01 * beta * tnorm[trip];
+  if ((threadIdx.x & 31) == 0)
+    bound[(long long)b * A.ntrip + trip] = A.mode == 2 ? 1.01 * beta : 1.01 * beta * tnorm[trip];
 }
 
 // relerr[b][pl][d] = bound[b][trip(pl)] / |delta[b][pl][d]|; trip(pl) = pl, or
@@ -310,35 +321,40 @@ extern "C" bs_status bs_mabs_error_bound(bs_plan p, double *bound_dev, const dou
   // NaN (all bits set) for every ring triple without a closed triangle
   EB_CUDA(cudaMemsetAsync(bound_dev, 0xFF, (size_t)out_batch * p->ntrip * sizeof(double), s));
   double *norms = p->at<double>(p->L.errn);
+  NormLevels N{};
+  BoundArgs B{};
+  B.nc = p->nc;
+  B.batch = p->chans ? p->batch : out_batch;
+  B.mode = p->chans ? 2 : p->general ? 1 : 0;
+  B.ntrip = p->ntrip;
   for (int li = 0; li < (int)p->levels.size(); ++li) {
     const Level &lv = p->levels[li];
-    if (lv.nslot == 0) continue;
     const long long m2 = (long long)lv.M * lv.M;
     const int nfield = p->batch * lv.nslot * p->nc;
-    k_field_norms<<<nfield, kNormThreads, 0, s>>>(p->at<float>(lv.offF), m2, norms);
-    EB_CUDA(cudaGetLastError());
-    BoundLevel B{};
-    B.norms = norms;
-    B.slot_of = p->at<int>(lv.offSlot);
-    B.kexp = prec == BS_PREC_SPLIT_FP16 ? p->at<int>(lv.offKexp) : nullptr;
-    B.level = li;
-    B.nslot = lv.nslot;
-    B.nc = p->nc;
-    B.batch = p->chans ? p->batch : out_batch;
-    B.mode = p->chans ? 2 : p->general ? 1 : 0;
-    B.ntrip = p->ntrip;
+    N.F[li] = p->at<float>(lv.offF);
+    N.m2[li] = m2;
+    N.first[li + 1] = N.first[li] + nfield;
+    BoundLevel &L = B.lev[li];
+    L.norms = norms + (size_t)N.first[li] * 3;
+    L.slot_of = p->at<int>(lv.offSlot);
+    L.kexp = prec == BS_PREC_SPLIT_FP16 ? p->at<int>(lv.offKexp) : nullptr;
+    L.nslot = lv.nslot;
     const double c_acc = prec == BS_PREC_FP32
                              ? (1024.0 + std::ceil((double)m2 / 1024.0) + 1.0) * kU
                              : 2.0 * kU * (3.0 * std::ceil((double)m2 / 16.0) + 1.0);
-    B.c1 = c_term + c_acc;
-    B.cf = (2.0 * (ceil_log2(lv.M) + 2) * 8.0 + 2.0) * kU;
-    B.floor16 = prec == BS_PREC_SPLIT_FP16 ? std::ldexp(1.0, -25) * (16384.0 + 128.0) * (double)m2
+    L.c1 = c_term + c_acc;
+    L.cf = (2.0 * (ceil_log2(lv.M) + 2) * 8.0 + 2.0) * kU;
+    L.floor16 = prec == BS_PREC_SPLIT_FP16 ? std::ldexp(1.0, -25) * (16384.0 + 128.0) * (double)m2
                                            : 0.0;
-    const int nt = B.batch * p->ntrip;
-    k_trip_bound<<<(nt + 255) / 256, 256, 0, s>>>(B, dtab, p->at<double>(p->L.tnorm),
-                                                  p->chans ? beta_int : bound_dev);
+  }
+  const int nfields = N.first[p->levels.size()];
+  if (nfields > 0) {
+    k_field_norms<<<nfields, kNormThreads, 0, s>>>(N, norms);
     EB_CUDA(cudaGetLastError());
-    norms += (size_t)nfield * 3;
+    const long long nt = 32LL * B.batch * p->ntrip;
+    k_trip_bound<<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(B, dtab, p->at<double>(p->L.tnorm),
+                                                              p->chans ? beta_int : bound_dev);
+    EB_CUDA(cudaGetLastError());
   }
   if (p->chans) {
     const int npl = closable ? (int)p->clos.size() : p->ntrip;
