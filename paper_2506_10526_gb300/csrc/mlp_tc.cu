@@ -20,12 +20,11 @@
 // (n-tiles 2kk, 2kk + 1) is exactly the A fragment of k-step kk of the next
 // layer, so activations stay in registers between the layers.
 //
-// Kernels (8 warps, 16 rows per warp, 128 rows per CTA):
-//   forward       h1 = tanh(W1 xn + b1), h2 = tanh(W2 h1 + b2), yn = w3.h2 + b3
-//   backward rows dz2 = dyn w3 (1 - h2^2), dz1 = (W2^T dz2)(1 - h1^2)
-//   wgrad         dW1 = dz1^T xn, dW2 = dz2^T h1 over a 128-row chunk per CTA
-//                 (operands staged transposed in shared memory), FP32 atomics
-//                 into the gradient; biases and the output layer in FP32.
+// Kernels:
+//   inference     h1 = tanh(W1 xn + b1), h2 = tanh(W2 h1 + b2), yn = w3.h2 + b3
+//   gradient      the same forward, dz2 = dyn w3 (1 - h2^2), dz1 = (W2^T dz2)(1 - h1^2),
+//                 dW1 = dz1^T xn, dW2 = dz2^T h1, in one kernel: nothing of a row
+//                 goes through global memory
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -40,7 +39,6 @@ namespace {
 constexpr int W = 128;           // hidden width of the tensor-core kernels
 constexpr int kWarps = 8, kThreads = 32 * kWarps, kRowsPerCta = 16 * kWarps;
 constexpr int LD2 = W + 8;       // bf16 pitch of the staged W2 (conflict-free fragments)
-constexpr int LDR = kRowsPerCta + 8;  // bf16 pitch of the transposed wgrad operands
 
 __device__ __forceinline__ uint32_t pack2(__nv_bfloat16 a, __nv_bfloat16 b) {
   return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
@@ -88,355 +86,6 @@ __device__ void stage_net(const MlpDev &M, __nv_bfloat16 *W1s, __nv_bfloat16 *W2
   for (int q = threadIdx.x; q < W; q += blockDim.x) w3[q] = __bfloat162float(__float2bfloat16_rn(p[q]));
 }
 
-// B fragment (k = 2t.., n = g) of a weight matrix stored [n][k] with pitch ld:
-// two consecutive k of one row, one 32-bit load
-__device__ __forceinline__ uint32_t bfrag_nk(const __nv_bfloat16 *Ws, int ld, int n, int k) {
-  return *reinterpret_cast<const uint32_t *>(Ws + n * ld + k);
-}
-
-// Forward for rows[r] = idx ? idx[r] : r.  y (denormalised) and, when store
-// is set, per row [xn (d) | h1 (W) | h2 (W) | yn].
-template <int K1>
-__global__ void __launch_bounds__(kThreads) k_mlp_tc_forward(MlpDev M, const float *__restrict__ x,
-                                                             int n, const int *__restrict__ idx,
-                                                             int nrows, float *__restrict__ y,
-                                                             float *__restrict__ store) {
-  constexpr int LD1 = K1 + 8, KS1 = K1 / 16;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __nv_bfloat16 *W1s = reinterpret_cast<__nv_bfloat16 *>(smem_raw);
-  __nv_bfloat16 *W2s = W1s + W * LD1;
-  float *b1 = reinterpret_cast<float *>(W2s + W * LD2), *b2 = b1 + W, *w3 = b2 + W;
-  stage_net<K1>(M, W1s, W2s, b1, b2, w3);
-  __syncthreads();
-  const int d = M.d, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int g = lane >> 2, t = lane & 3;
-  // the warp's rows g and g + 8
-  const int r0 = blockIdx.x * kRowsPerCta + warp * 16 + g, r1 = r0 + 8;
-  int row0 = -1, row1 = -1;
-  if (r0 < nrows) row0 = idx ? idx[r0] : r0;
-  if (r1 < nrows) row1 = idx ? idx[r1] : r1;
-  const bool ok0 = row0 >= 0 && row0 < n, ok1 = row1 >= 0 && row1 < n;
-  const float *mu = M.norm, *sd = M.norm + d;
-  const int sw = d + 2 * W + 1;
-  float *st0 = (store && ok0) ? store + (long long)r0 * sw : nullptr;
-  float *st1 = (store && ok1) ? store + (long long)r1 * sw : nullptr;
-  // layer 1: A = xn (hi, lo), B = W1^T
-  float c[16][4];
-#pragma unroll
-  for (int j = 0; j < 16; ++j) c[j][0] = c[j][1] = c[j][2] = c[j][3] = 0.f;
-#pragma unroll
-  for (int kk = 0; kk < KS1; ++kk) {
-    float v[8];  // (row, col): (g, 2t), (g, 2t+1), (g+8, 2t), (g+8, 2t+1), then cols + 8
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int col = 16 * kk + 2 * t + (q & 1) + ((q >> 2) << 3);
-      const bool hi_row = (q >> 1) & 1;
-      const bool okr = hi_row ? ok1 : ok0;
-      const int row = hi_row ? row1 : row0;
-      float xv = 0.f;
-      if (okr && col < d) {
-        xv = (x[(long long)row * d + col] - mu[col]) / sd[col];
-        float *st = hi_row ? st1 : st0;
-        if (st) st[col] = xv;
-      }
-      v[q] = xv;
-    }
-    uint32_t ah[4], al[4];
-    split2(v[0], v[1], ah[0], al[0]);
-    split2(v[2], v[3], ah[1], al[1]);
-    split2(v[4], v[5], ah[2], al[2]);
-    split2(v[6], v[7], ah[3], al[3]);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const uint32_t b0 = bfrag_nk(W1s, LD1, 8 * j + g, 16 * kk + 2 * t);
-      const uint32_t bb = bfrag_nk(W1s, LD1, 8 * j + g, 16 * kk + 2 * t + 8);
-      mma16816(c[j], ah, b0, bb);
-      mma16816(c[j], al, b0, bb);
-    }
-  }
-  // h1 = tanh(z1 + b1) -> A fragments of layer 2
-  uint32_t a2h[8][4], a2l[8][4];
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const int col = 8 * j + 2 * t;
-    const float h00 = tanhf(c[j][0] + b1[col]), h01 = tanhf(c[j][1] + b1[col + 1]);
-    const float h10 = tanhf(c[j][2] + b1[col]), h11 = tanhf(c[j][3] + b1[col + 1]);
-    if (st0) {
-      st0[d + col] = h00;
-      st0[d + col + 1] = h01;
-    }
-    if (st1) {
-      st1[d + col] = h10;
-      st1[d + col + 1] = h11;
-    }
-    const int kk = j >> 1, hs = (j & 1) * 2;  // n-tile 2kk -> a0, a1; 2kk + 1 -> a2, a3
-    split2(h00, h01, a2h[kk][hs], a2l[kk][hs]);
-    split2(h10, h11, a2h[kk][hs + 1], a2l[kk][hs + 1]);
-  }
-  // layer 2 in two halves of 8 n-tiles; yn accumulates on the fly
-  float y0 = 0.f, y1 = 0.f;
-#pragma unroll
-  for (int half = 0; half < 2; ++half) {
-    float c2[8][4];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) c2[j][0] = c2[j][1] = c2[j][2] = c2[j][3] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < 8; ++kk) {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int nrow = 8 * (8 * half + j) + g;
-        const uint32_t b0 = bfrag_nk(W2s, LD2, nrow, 16 * kk + 2 * t);
-        const uint32_t bb = bfrag_nk(W2s, LD2, nrow, 16 * kk + 2 * t + 8);
-        mma16816(c2[j], a2h[kk], b0, bb);
-        mma16816(c2[j], a2l[kk], b0, bb);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int col = 8 * (8 * half + j) + 2 * t;
-      const float h00 = tanhf(c2[j][0] + b2[col]), h01 = tanhf(c2[j][1] + b2[col + 1]);
-      const float h10 = tanhf(c2[j][2] + b2[col]), h11 = tanhf(c2[j][3] + b2[col + 1]);
-      y0 = fmaf(w3[col], h00, fmaf(w3[col + 1], h01, y0));
-      y1 = fmaf(w3[col], h10, fmaf(w3[col + 1], h11, y1));
-      if (st0) {
-        st0[d + W + col] = h00;
-        st0[d + W + col + 1] = h01;
-      }
-      if (st1) {
-        st1[d + W + col] = h10;
-        st1[d + W + col + 1] = h11;
-      }
-    }
-  }
-  // the four threads of a group hold the row's partial dot products
-  y0 += __shfl_xor_sync(0xffffffffu, y0, 1);
-  y0 += __shfl_xor_sync(0xffffffffu, y0, 2);
-  y1 += __shfl_xor_sync(0xffffffffu, y1, 1);
-  y1 += __shfl_xor_sync(0xffffffffu, y1, 2);
-  if (t == 0) {
-    const float b3 = M.p[(long long)W * d + W + W * W + W + W];
-    const float yn0 = y0 + b3, yn1 = y1 + b3;
-    const float my = M.norm[2 * d], sy = M.norm[2 * d + 1];
-    if (ok0) {
-      if (st0) st0[d + 2 * W] = yn0;
-      if (y) y[r0] = my + sy * yn0;
-    }
-    if (ok1) {
-      if (st1) st1[d + 2 * W] = yn1;
-      if (y) y[r1] = my + sy * yn1;
-    }
-  }
-}
-
-// Per-row backward: dyn = 2 (yn - tn) / nrows, dz2 = dyn w3 (1 - h2^2),
-// dz1 = (W2^T dz2)(1 - h1^2).  bw rows [dz1 (W) | dz2 (W) | dyn]; loss += mean
-// of squared residuals.
-__global__ void __launch_bounds__(kThreads) k_mlp_tc_backward_rows(
-    MlpDev M, const float *__restrict__ tgt, const int *__restrict__ idx, int nrows,
-    const float *__restrict__ store, float *__restrict__ bw, float *__restrict__ loss) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __nv_bfloat16 *W2s = reinterpret_cast<__nv_bfloat16 *>(smem_raw);  // [j][k], pitch LD2
-  float *w3 = reinterpret_cast<float *>(W2s + W * LD2);
-  const int d = M.d;
-  {
-    const float *p = M.p + (long long)W * d + W;
-    for (int q = threadIdx.x; q < W * W; q += blockDim.x) {
-      const int j = q / W, k = q - j * W;
-      W2s[j * LD2 + k] = __float2bfloat16_rn(p[q]);
-    }
-    for (int q = threadIdx.x; q < W; q += blockDim.x)
-      w3[q] = __bfloat162float(__float2bfloat16_rn(p[W * W + W + q]));
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int g = lane >> 2, t = lane & 3;
-  const int r0 = blockIdx.x * kRowsPerCta + warp * 16 + g, r1 = r0 + 8;
-  const bool ok0 = r0 < nrows, ok1 = r1 < nrows;
-  const int sw = d + 2 * W + 1, bwid = 2 * W + 1;
-  const float *s0 = store + (long long)(ok0 ? r0 : 0) * sw;
-  const float *s1 = store + (long long)(ok1 ? r1 : 0) * sw;
-  float *o0 = bw + (long long)(ok0 ? r0 : 0) * bwid;
-  float *o1 = bw + (long long)(ok1 ? r1 : 0) * bwid;
-  const float my = M.norm[2 * d], sy = M.norm[2 * d + 1];
-  float dyn0 = 0.f, dyn1 = 0.f, l2 = 0.f;
-  if (ok0) {
-    const float res = s0[d + 2 * W] - (tgt[idx ? idx[r0] : r0] - my) / sy;
-    dyn0 = 2.f * res / (float)nrows;
-    if (t == 0) l2 += res * res;
-  }
-  if (ok1) {
-    const float res = s1[d + 2 * W] - (tgt[idx ? idx[r1] : r1] - my) / sy;
-    dyn1 = 2.f * res / (float)nrows;
-    if (t == 0) l2 += res * res;
-  }
-  // dz2 in A-fragment order (k-step kk covers j = 16 kk .. 16 kk + 15)
-  uint32_t ah[8][4], al[8][4];
-#pragma unroll
-  for (int kk = 0; kk < 8; ++kk) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {  // a0: (g, 2t), a1: (g+8, 2t), a2: (g, 2t+8), a3: (g+8, 2t+8)
-      const int j = 16 * kk + 2 * t + ((q >> 1) << 3);
-      const bool hi_row = q & 1;
-      const float *sr = hi_row ? s1 : s0;
-      const float dyn = hi_row ? dyn1 : dyn0;
-      const bool okr = hi_row ? ok1 : ok0;
-      float z0 = 0.f, z1 = 0.f;
-      if (okr) {
-        const float h0 = sr[d + W + j], h1 = sr[d + W + j + 1];
-        z0 = dyn * w3[j] * (1.f - h0 * h0);
-        z1 = dyn * w3[j + 1] * (1.f - h1 * h1);
-        float *o = hi_row ? o1 : o0;
-        o[W + j] = z0;
-        o[W + j + 1] = z1;
-      }
-      split2(z0, z1, ah[kk][q], al[kk][q]);
-    }
-  }
-  // dz1 pre-activation: sum_j dz2_j W2[j][k]; B = W2 as (K = j) x (N = k), two
-  // 16-bit loads per register (consecutive j are a row apart)
-#pragma unroll
-  for (int half = 0; half < 2; ++half) {
-    float c[8][4];
-#pragma unroll
-    for (int n = 0; n < 8; ++n) c[n][0] = c[n][1] = c[n][2] = c[n][3] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < 8; ++kk) {
-#pragma unroll
-      for (int n = 0; n < 8; ++n) {
-        const int kcol = 8 * (8 * half + n) + g;
-        const int j = 16 * kk + 2 * t;
-        const uint32_t b0 = pack2(W2s[j * LD2 + kcol], W2s[(j + 1) * LD2 + kcol]);
-        const uint32_t bb = pack2(W2s[(j + 8) * LD2 + kcol], W2s[(j + 9) * LD2 + kcol]);
-        mma16816(c[n], ah[kk], b0, bb);
-        mma16816(c[n], al[kk], b0, bb);
-      }
-    }
-#pragma unroll
-    for (int n = 0; n < 8; ++n) {
-      const int k = 8 * (8 * half + n) + 2 * t;
-      if (ok0) {
-        const float h0 = s0[d + k], h1 = s0[d + k + 1];
-        o0[k] = c[n][0] * (1.f - h0 * h0);
-        o0[k + 1] = c[n][1] * (1.f - h1 * h1);
-      }
-      if (ok1) {
-        const float h0 = s1[d + k], h1 = s1[d + k + 1];
-        o1[k] = c[n][2] * (1.f - h0 * h0);
-        o1[k + 1] = c[n][3] * (1.f - h1 * h1);
-      }
-    }
-  }
-  if (t == 0) {
-    if (ok0) o0[2 * W] = dyn0;
-    if (ok1) o1[2 * W] = dyn1;
-  }
-  for (int off = 16; off > 0; off >>= 1) l2 += __shfl_xor_sync(0xffffffffu, l2, off);
-  if (loss && lane == 0) atomicAdd(loss, l2 / (float)nrows);
-}
-
-// Weight gradients over one 128-row chunk: blockIdx.y = 0: dW1 = dz1^T xn and
-// db1; 1: dW2 = dz2^T h1, db2, and the output layer dw3 = dyn^T h2, db3 (FP32).
-// A = dz^T [W][r] and B = in^T [KN][r] are staged in shared memory, r
-// contiguous, as BF16 hi / lo.
-template <int K1>
-__global__ void __launch_bounds__(kThreads) k_mlp_tc_wgrad(MlpDev M, int nrows,
-                                                           const float *__restrict__ store,
-                                                           const float *__restrict__ bw) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int layer = blockIdx.y;
-  const int d = M.d;
-  const int KN = layer == 0 ? K1 : W;  // inputs of the layer (padded)
-  __nv_bfloat16 *Ah = reinterpret_cast<__nv_bfloat16 *>(smem_raw);
-  __nv_bfloat16 *Al = Ah + W * LDR;
-  __nv_bfloat16 *Bh = Al + W * LDR;
-  __nv_bfloat16 *Bl = Bh + KN * LDR;
-  const int r0 = blockIdx.x * kRowsPerCta;
-  const int sw = d + 2 * W + 1, bwid = 2 * W + 1;
-  float *gW1 = M.g, *gb1 = gW1 + W * d, *gW2 = gb1 + W, *gb2 = gW2 + W * W, *gw3 = gb2 + W,
-        *gb3 = gw3 + W;
-  const int zoff = layer == 0 ? 0 : W, ioff = layer == 0 ? 0 : d;
-  // stage dz^T (and the bias sums: each thread keeps one j)
-  float bsum = 0.f;
-  for (int e = threadIdx.x; e < kRowsPerCta * W; e += blockDim.x) {
-    const int r = e / W, j = e - r * W;
-    const float z = (r0 + r < nrows) ? bw[(long long)(r0 + r) * bwid + zoff + j] : 0.f;
-    bsum += z;
-    const __nv_bfloat16 h = __float2bfloat16_rn(z);
-    Ah[j * LDR + r] = h;
-    Al[j * LDR + r] = __float2bfloat16_rn(z - __bfloat162float(h));
-  }
-  atomicAdd((layer == 0 ? gb1 : gb2) + (threadIdx.x % W), bsum);
-  for (int e = threadIdx.x; e < kRowsPerCta * KN; e += blockDim.x) {
-    const int r = e / KN, k = e - r * KN;
-    const bool live = r0 + r < nrows && (layer == 1 || k < d);
-    const float v = live ? store[(long long)(r0 + r) * sw + ioff + k] : 0.f;
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    Bh[k * LDR + r] = h;
-    Bl[k * LDR + r] = __float2bfloat16_rn(v - __bfloat162float(h));
-  }
-  if (layer == 1 && threadIdx.x < W) {  // output layer, FP32
-    const int k = threadIdx.x;
-    float acc = 0.f, db = 0.f;
-    for (int r = r0; r < min(nrows, r0 + kRowsPerCta); ++r) {
-      const float dyn = bw[(long long)r * bwid + 2 * W];
-      acc = fmaf(dyn, store[(long long)r * sw + d + W + k], acc);
-      db += dyn;
-    }
-    atomicAdd(gw3 + k, acc);
-    if (k == 0) atomicAdd(gb3, db);
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int g = lane >> 2, t = lane & 3;
-  const int jr = 16 * warp + g;  // output rows jr, jr + 8
-  float c[W / 8][4];
-#pragma unroll
-  for (int n = 0; n < W / 8; ++n) c[n][0] = c[n][1] = c[n][2] = c[n][3] = 0.f;
-  const int NT = KN / 8;
-#pragma unroll
-  for (int kk = 0; kk < kRowsPerCta / 16; ++kk) {
-    const int rc = 16 * kk + 2 * t;
-    uint32_t ah[4], al[4];
-    ah[0] = *reinterpret_cast<const uint32_t *>(Ah + jr * LDR + rc);
-    ah[1] = *reinterpret_cast<const uint32_t *>(Ah + (jr + 8) * LDR + rc);
-    ah[2] = *reinterpret_cast<const uint32_t *>(Ah + jr * LDR + rc + 8);
-    ah[3] = *reinterpret_cast<const uint32_t *>(Ah + (jr + 8) * LDR + rc + 8);
-    al[0] = *reinterpret_cast<const uint32_t *>(Al + jr * LDR + rc);
-    al[1] = *reinterpret_cast<const uint32_t *>(Al + (jr + 8) * LDR + rc);
-    al[2] = *reinterpret_cast<const uint32_t *>(Al + jr * LDR + rc + 8);
-    al[3] = *reinterpret_cast<const uint32_t *>(Al + (jr + 8) * LDR + rc + 8);
-#pragma unroll
-    for (int n = 0; n < W / 8; ++n) {
-      if (n < NT) {
-        const int kb = (8 * n + g) * LDR + rc;
-        const uint32_t bh0 = *reinterpret_cast<const uint32_t *>(Bh + kb);
-        const uint32_t bh1 = *reinterpret_cast<const uint32_t *>(Bh + kb + 8);
-        const uint32_t bl0 = *reinterpret_cast<const uint32_t *>(Bl + kb);
-        const uint32_t bl1 = *reinterpret_cast<const uint32_t *>(Bl + kb + 8);
-        mma16816(c[n], ah, bh0, bh1);
-        mma16816(c[n], ah, bl0, bl1);
-        mma16816(c[n], al, bh0, bh1);
-      }
-    }
-  }
-  float *gW = layer == 0 ? gW1 : gW2;
-  const int ldw = layer == 0 ? d : W;
-#pragma unroll
-  for (int n = 0; n < W / 8; ++n) {
-    if (n < NT) {
-      const int k = 8 * n + 2 * t;
-      if (k < ldw) {
-        atomicAdd(gW + jr * ldw + k, c[n][0]);
-        atomicAdd(gW + (jr + 8) * ldw + k, c[n][2]);
-      }
-      if (k + 1 < ldw) {
-        atomicAdd(gW + jr * ldw + k + 1, c[n][1]);
-        atomicAdd(gW + (jr + 8) * ldw + k + 1, c[n][3]);
-      }
-    }
-  }
-}
-
 // ------------------------------------------------------------- inference
 //
 // Packed FP32 pairs: one instruction for two values.
@@ -475,14 +124,19 @@ __device__ __forceinline__ float rcp(float x) {
 // (1 - e) / (1 + e) with e = exp(-2 |x|) <= 1/3, no cancellation; below: an odd
 // polynomial |x| + |x|^3 P(x^2), P a degree-4 Chebyshev least-squares fit on
 // [0, 0.55^2] (relative error of the fit 1.1e-9).  Within 3e-7 relative of tanh
-// everywhere; NaN stays NaN, infinities give 1.
+// everywhere; NaN stays NaN, infinities give 1.  CORR: one more step takes the
+// reciprocal's error out of the quotient, for the gradient (1 - tanh^2), where an
+// error of one sign adds up over the rows; 7% of the inference time.
+template <bool CORR = false>
 __device__ __forceinline__ void tanh_pair(float x0, float x1, float &y0, float &y1) {
   const float a0 = fabsf(x0), a1 = fabsf(x1);
   const uint64_t a = pk(a0, a1), one = pk(1.f, 1.f);
   const uint64_t u = mul2(a, pk(-2.88539008f, -2.88539008f));  // -2 log2(e) |x|
   const uint64_t e = pk(ex2(lo_f(u)), ex2(hi_f(u)));
   const uint64_t den = add2(e, one);
-  const uint64_t big = mul2(fma2(e, pk(-1.f, -1.f), one), pk(rcp(lo_f(den)), rcp(hi_f(den))));
+  const uint64_t num = fma2(e, pk(-1.f, -1.f), one), rd = pk(rcp(lo_f(den)), rcp(hi_f(den)));
+  uint64_t big = mul2(num, rd);
+  if constexpr (CORR) big = fma2(fma2(big, pk(-lo_f(den), -hi_f(den)), num), rd, big);
   const uint64_t q = mul2(a, a);
   uint64_t p = fma2(q, pk(-0.00626437f, -0.00626437f), pk(0.02106414f, 0.02106414f));
   p = fma2(q, p, pk(-0.0538503f, -0.0538503f));
@@ -515,7 +169,7 @@ __device__ __forceinline__ uint32_t b_addr(uint32_t base, int ld, int j, int kk,
 // tensor pipe or HBM: the kernel it replaced issued 5970 warp instructions per 16
 // rows (weights staged for every 128 rows, one 32-bit shared load per B register,
 // a division per input, the library tanh on two divergent branches) and kept the
-// issue slots 47% busy.  1540 x 60^2 rows: 1.91 ms, 3.71 ms before.
+// issue slots 47% busy.  1540 x 60^2 rows: 1.85 ms, 3.71 ms before.
 template <int K1>
 __global__ void __launch_bounds__(kThreads, 2) k_mlp_tc_infer(MlpDev M, const float *__restrict__ x,
                                                               int n, float *__restrict__ y) {
@@ -584,16 +238,15 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp_tc_infer(MlpDev M, const fl
         c[j][1] = c[j][3] = b.y;
       }
 #pragma unroll
-      for (int kk = 0; kk < KS1; ++kk)
+      for (int kk = 0; kk < KS1; ++kk) {
+        uint32_t r[4][4];
 #pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-          uint32_t r[4];
-          ldsm4(r, b_addr(a1, LD1, 8 * half + j, kk, lane));
-          mma16816(c[j], ah[kk], r[0], r[1]);
-          mma16816(c[j + 1], ah[kk], r[2], r[3]);
-          mma16816(c[j], al[kk], r[0], r[1]);
-          mma16816(c[j + 1], al[kk], r[2], r[3]);
-        }
+        for (int j = 0; j < 4; ++j) ldsm4(r[j], b_addr(a1, LD1, 8 * half + 2 * j, kk, lane));
+#pragma unroll
+        for (int j = 0; j < 8; ++j) mma16816(c[j], ah[kk], r[j / 2][2 * (j & 1)], r[j / 2][2 * (j & 1) + 1]);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) mma16816(c[j], al[kk], r[j / 2][2 * (j & 1)], r[j / 2][2 * (j & 1) + 1]);
+      }
       // h1 = tanh(z1): n-tile 2kk -> a0, a1 of k-step kk; 2kk + 1 -> a2, a3
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
@@ -616,16 +269,15 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp_tc_infer(MlpDev M, const fl
         c[j][1] = c[j][3] = b.y;
       }
 #pragma unroll
-      for (int kk = 0; kk < 8; ++kk)
+      for (int kk = 0; kk < 8; ++kk) {
+        uint32_t r[2][4];
 #pragma unroll
-        for (int j = 0; j < 4; j += 2) {
-          uint32_t r[4];
-          ldsm4(r, b_addr(a2, LD2, 4 * qt + j, kk, lane));
-          mma16816(c[j], h1h[kk], r[0], r[1]);
-          mma16816(c[j + 1], h1h[kk], r[2], r[3]);
-          mma16816(c[j], h1l[kk], r[0], r[1]);
-          mma16816(c[j + 1], h1l[kk], r[2], r[3]);
-        }
+        for (int j = 0; j < 2; ++j) ldsm4(r[j], b_addr(a2, LD2, 4 * qt + 2 * j, kk, lane));
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mma16816(c[j], h1h[kk], r[j / 2][2 * (j & 1)], r[j / 2][2 * (j & 1) + 1]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mma16816(c[j], h1l[kk], r[j / 2][2 * (j & 1)], r[j / 2][2 * (j & 1) + 1]);
+      }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const float2 w = *reinterpret_cast<const float2 *>(w3 + 8 * (4 * qt + j) + 2 * t);
@@ -647,21 +299,463 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp_tc_infer(MlpDev M, const fl
   }
 }
 
-template <int K1>
-size_t fwd_smem_tc() {
-  return (size_t)W * (K1 + 8) * 2 + (size_t)W * LD2 * 2 + 3 * W * sizeof(float);
+// ------------------------------------------------------------- gradient
+//
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
 }
-size_t bwd_smem_tc() { return (size_t)W * LD2 * 2 + W * sizeof(float); }
-size_t wgrad_smem_tc() { return (size_t)4 * W * LDR * 2; }
+__device__ __forceinline__ void ldsm2t(uint32_t (&r)[2], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+               : "=r"(r[0]), "=r"(r[1])
+               : "r"(addr));
+}
 
+constexpr int kGradRows = 64, kGradThreads = 512;
+
+// Floats from one partial gradient to the next (the parameters, padded to 16 bytes).
+__host__ __device__ constexpr int part_stride(int d) {
+  return (W * d + W + W * W + W + W + 1 + 3) / 4 * 4;
+}
+// The network as the gradient kernel stages it: W1 [W][K1 + 8] and W2 [W][LD2] in BF16,
+// then b1, b2, w3 (BF16-rounded), in one block of 16-byte pieces.
+constexpr int image_bytes(int k1) { return W * (k1 + 8) * 2 + W * LD2 * 2 + 3 * W * 4; }
+// Parameter q's value into the image (b3 is read from the parameters).
+__device__ __forceinline__ void image_put(unsigned char *im, int d, int k1, int q, float v) {
+  __nv_bfloat16 *W1 = reinterpret_cast<__nv_bfloat16 *>(im), *W2 = W1 + W * (k1 + 8);
+  float *vec = reinterpret_cast<float *>(W2 + W * LD2);
+  if (q < W * d) {
+    const int j = q / d;
+    W1[j * (k1 + 8) + q - j * d] = __float2bfloat16_rn(v);
+    return;
+  }
+  q -= W * d;
+  if (q < W) {
+    vec[q] = v;
+    return;
+  }
+  q -= W;
+  if (q < W * W) {
+    W2[(q / W) * LD2 + q % W] = __float2bfloat16_rn(v);
+    return;
+  }
+  q -= W * W;
+  if (q < W)
+    vec[W + q] = v;
+  else if (q < 2 * W)
+    vec[W + q] = __bfloat162float(__float2bfloat16_rn(v));
+}
+__global__ void k_mlp_tc_image(MlpDev M, int k1, int np, unsigned char *__restrict__ im) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < np) image_put(im, M.d, k1, q, M.p[q]);
+}
+
+// Shared memory of the gradient kernel (BF16 tiles row major, FP32 vectors).
 template <int K1>
-cudaError_t forward_k(const MlpDev &M, const float *x, int n, const int *idx, int nrows, float *y,
-                      float *store, cudaStream_t s) {
-  cudaError_t e = smem_optin_once<k_mlp_tc_forward<K1>>();
-  if (e != cudaSuccess) return e;
-  k_mlp_tc_forward<K1><<<(nrows + kRowsPerCta - 1) / kRowsPerCta, kThreads, fwd_smem_tc<K1>(), s>>>(
-      M, x, n, idx, nrows, y, store);
-  return cudaGetLastError();
+struct GradLay {
+  static constexpr int LD1 = K1 + 8;
+  static constexpr int W1s = 0, W2s = W1s + W * LD1 * 2, net = W2s + W * LD2 * 2;
+  static constexpr int X = net + 3 * W * 4;             // hi, lo [64][LD1]
+  static constexpr int H1 = X + 2 * kGradRows * LD1 * 2;  // hi, lo [64][LD2]
+  static constexpr int Z2 = H1 + 2 * kGradRows * LD2 * 2, Z1 = Z2 + 2 * kGradRows * LD2 * 2;
+  static constexpr int vec = Z1 + 2 * kGradRows * LD2 * 2;
+  // gb1, gb2, gw3 [4][W], mu, inv [K1], yn parts [4][64], tn, ok [64], row [64], gb3
+  static constexpr int bytes = vec + (12 * W + 2 * K1 + 4 * kGradRows + 3 * kGradRows + 4) * 4;
+};
+
+// Loss and gradient of nrows rows (drawn as k_mlp_sample draws them when seeded:
+// row r of step `step` is mix(seed, step, r) mod n) as one partial gradient per CTA,
+// part[CTA][np], summed by k_mlp_tc_reduce; loss += mean of squared residuals.
+//
+// A tile of 64 rows takes the 16 warps through five MMA passes (forward 1 and 2,
+// dz1, dW2, dW1) with its activations in shared memory: warp w has rows 16 (w % 4)
+// and outputs 32 (w / 4) of the per-row passes, and keeps a 16 x 64 block of dW2
+// and a 16 x K1/2 block of dW1 in registers over all its tiles.  Transposed operands
+// (W2^T, dz^T, h1, xn by rows) come out of the row-major tiles with
+// ldmatrix.trans.
+//
+// The three kernels it replaced wrote 559 floats a row to global memory and read
+// them back, ran a batch of 8192 rows on 64 of the 152 SMs, staged the weights in
+// each, transposed through strided 16-bit stores and added every CTA's 22 thousand
+// weights with atomics.  24 steps of 8192 rows and one gradient of 122880 (d = 45): 2.43 ms in
+// those kernels, 0.65 here (with k_mlp_tc_reduce).
+template <int K1>
+__global__ void __launch_bounds__(kGradThreads, 1)
+    k_mlp_tc_grad(MlpDev M, const float *__restrict__ x, const float *__restrict__ tgt, int n,
+                  int nrows, int sampled, unsigned long long seed, int step,
+                  const unsigned char *__restrict__ im, float *__restrict__ part,
+                  float *__restrict__ loss) {
+  using Ly = GradLay<K1>;
+  constexpr int LD1 = K1 + 8, KS1 = K1 / 16, NT1 = K1 / 16;  // dW1 n-tiles of a warp
+  static_assert(part_stride(K1) * 4 <= Ly::vec - Ly::X, "the partial gradient over the tile's buffers");
+  extern __shared__ __align__(16) unsigned char sm[];
+  const float *b1 = reinterpret_cast<const float *>(sm + Ly::net), *b2 = b1 + W, *w3 = b2 + W;
+  float *gb1 = reinterpret_cast<float *>(sm + Ly::vec), *gb2 = gb1 + 4 * W, *gw3 = gb2 + 4 * W, *mu = gw3 + 4 * W, *inv = mu + K1;
+  float *ypart = inv + K1, *tn = ypart + 4 * kGradRows, *okr = tn + kGradRows;
+  int *rowid = reinterpret_cast<int *>(okr + kGradRows);
+  float *gb3 = reinterpret_cast<float *>(rowid + kGradRows);
+  const int d = M.d, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = lane >> 2, t = lane & 3;
+  const int rg = warp & 3, cq = warp >> 2;   // per-row passes: rows 16 rg.., outputs 32 cq..
+  const int jb = warp & 7, kb = warp >> 3;   // weight gradients: rows 16 jb.., half kb of the inputs
+  const uint32_t sb = (uint32_t)__cvta_generic_to_shared(sm);
+  const uint32_t aW1 = sb + Ly::W1s, aW2 = sb + Ly::W2s;
+  for (int q = tid; q < (Ly::net + 3 * W * 4) / 16; q += kGradThreads)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sb + 16u * q), "l"(im + 16 * q)
+                 : "memory");
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  for (int q = tid; q < 12 * W; q += kGradThreads) gb1[q] = 0.f;
+  if (tid == 0) *gb3 = 0.f;
+  for (int k = tid; k < K1; k += kGradThreads) {
+    mu[k] = k < d ? M.norm[k] : 0.f;
+    inv[k] = k < d ? 1.f / M.norm[d + k] : 0.f;
+  }
+  const float b3 = M.p[(long long)W * d + W + W * W + W + W];
+  const float my = M.norm[2 * d], sy = M.norm[2 * d + 1];
+  float l2 = 0.f, sdy = 0.f;  // sums of squared residuals and of dyn
+  float gW2[8][4], gW1[NT1][4];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) gW2[j][0] = gW2[j][1] = gW2[j][2] = gW2[j][3] = 0.f;
+#pragma unroll
+  for (int j = 0; j < NT1; ++j) gW1[j][0] = gW1[j][1] = gW1[j][2] = gW1[j][3] = 0.f;
+
+  // lane offsets (elements) of the 8x8 matrices of an ldmatrix.x4
+  const int aro = lane & 15, aco = (lane >> 4) << 3;                       // A: rows, then k + 8
+  const int tro = (lane & 7) + ((lane >> 4) << 3), tco = lane & 8;         // A^T from [k][m]
+  const int bro = lane & 15, bco = (lane >> 4) << 3;                       // B from [k][n]: two n-tiles
+  auto a_at = [&](uint32_t buf, int ld, int r0, int kk) {
+    return buf + 2u * (uint32_t)((r0 + aro) * ld + 16 * kk + aco);
+  };
+
+  const int ntile = (nrows - 1) / kGradRows + 1;
+  for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    __syncthreads();  // the previous tile's readers are done
+    if (tid < kGradRows) {
+      const int r = tile * kGradRows + tid;
+      int row = -1;
+      if (r < nrows) row = sampled ? mlp_sample_row(seed, step, r, n) : r;
+      rowid[tid] = row;
+      okr[tid] = row >= 0 ? 1.f : 0.f;
+      tn[tid] = row >= 0 ? (tgt[row] - my) / sy : 0.f;
+    }
+    __syncthreads();
+    for (int q = tid; q < kGradRows * (K1 / 2); q += kGradThreads) {
+      const int r = q / (K1 / 2), c = 2 * (q - r * (K1 / 2)), row = rowid[r];
+      float v0 = 0.f, v1 = 0.f;
+      if (row >= 0) {
+        const float *xr = x + (long long)row * d;
+        if (c < d) v0 = (xr[c] - mu[c]) * inv[c];
+        if (c + 1 < d) v1 = (xr[c + 1] - mu[c + 1]) * inv[c + 1];
+      }
+      uint32_t hi, lo;
+      split2(v0, v1, hi, lo);
+      *reinterpret_cast<uint32_t *>(sm + Ly::X + 2 * (r * LD1 + c)) = hi;
+      *reinterpret_cast<uint32_t *>(sm + Ly::X + 2 * (kGradRows * LD1 + r * LD1 + c)) = lo;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");  // the network (first tile)
+    __syncthreads();
+    // ---- forward 1
+    float h1[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 b = *reinterpret_cast<const float2 *>(b1 + 32 * cq + 8 * j + 2 * t);
+      h1[j][0] = h1[j][2] = b.x;
+      h1[j][1] = h1[j][3] = b.y;
+    }
+#pragma unroll
+    for (int kk = 0; kk < KS1; ++kk) {
+      uint32_t ah[4], al[4], r0[4], r1[4];
+      ldsm4(ah, a_at(sb + Ly::X, LD1, 16 * rg, kk));
+      ldsm4(al, a_at(sb + Ly::X + 2 * kGradRows * LD1, LD1, 16 * rg, kk));
+      ldsm4(r0, b_addr(aW1, LD1, 4 * cq, kk, lane));
+      ldsm4(r1, b_addr(aW1, LD1, 4 * cq + 2, kk, lane));
+      mma16816(h1[0], ah, r0[0], r0[1]);
+      mma16816(h1[1], ah, r0[2], r0[3]);
+      mma16816(h1[2], ah, r1[0], r1[1]);
+      mma16816(h1[3], ah, r1[2], r1[3]);
+      mma16816(h1[0], al, r0[0], r0[1]);
+      mma16816(h1[1], al, r0[2], r0[3]);
+      mma16816(h1[2], al, r1[0], r1[1]);
+      mma16816(h1[3], al, r1[2], r1[3]);
+    }
+    // a C tile's pair (row, columns 2t, 2t + 1) into a row-major hi / lo tile
+    auto put = [&](int buf, int j, const float (&c)[4]) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        uint32_t hi, lo;
+        split2(c[2 * q], c[2 * q + 1], hi, lo);
+        const int o = (16 * rg + g + 8 * q) * LD2 + 32 * cq + 8 * j + 2 * t;
+        *reinterpret_cast<uint32_t *>(sm + buf + 2 * o) = hi;
+        *reinterpret_cast<uint32_t *>(sm + buf + 2 * (kGradRows * LD2 + o)) = lo;
+      }
+    };
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      tanh_pair<true>(h1[j][0], h1[j][1], h1[j][0], h1[j][1]);
+      tanh_pair<true>(h1[j][2], h1[j][3], h1[j][2], h1[j][3]);
+      put(Ly::H1, j, h1[j]);
+    }
+    __syncthreads();
+    // ---- forward 2 and the output
+    float c2[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 b = *reinterpret_cast<const float2 *>(b2 + 32 * cq + 8 * j + 2 * t);
+      c2[j][0] = c2[j][2] = b.x;
+      c2[j][1] = c2[j][3] = b.y;
+    }
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk) {
+      uint32_t ah[4], al[4], r0[4], r1[4];
+      ldsm4(ah, a_at(sb + Ly::H1, LD2, 16 * rg, kk));
+      ldsm4(al, a_at(sb + Ly::H1 + 2 * kGradRows * LD2, LD2, 16 * rg, kk));
+      ldsm4(r0, b_addr(aW2, LD2, 4 * cq, kk, lane));
+      ldsm4(r1, b_addr(aW2, LD2, 4 * cq + 2, kk, lane));
+      mma16816(c2[0], ah, r0[0], r0[1]);
+      mma16816(c2[1], ah, r0[2], r0[3]);
+      mma16816(c2[2], ah, r1[0], r1[1]);
+      mma16816(c2[3], ah, r1[2], r1[3]);
+      mma16816(c2[0], al, r0[0], r0[1]);
+      mma16816(c2[1], al, r0[2], r0[3]);
+      mma16816(c2[2], al, r1[0], r1[1]);
+      mma16816(c2[3], al, r1[2], r1[3]);
+    }
+    float y0 = 0.f, y1 = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 w = *reinterpret_cast<const float2 *>(w3 + 32 * cq + 8 * j + 2 * t);
+      tanh_pair<true>(c2[j][0], c2[j][1], c2[j][0], c2[j][1]);
+      tanh_pair<true>(c2[j][2], c2[j][3], c2[j][2], c2[j][3]);
+      y0 = fmaf(w.x, c2[j][0], fmaf(w.y, c2[j][1], y0));
+      y1 = fmaf(w.x, c2[j][2], fmaf(w.y, c2[j][3], y1));
+    }
+    y0 += __shfl_xor_sync(0xffffffffu, y0, 1);
+    y0 += __shfl_xor_sync(0xffffffffu, y0, 2);
+    y1 += __shfl_xor_sync(0xffffffffu, y1, 1);
+    y1 += __shfl_xor_sync(0xffffffffu, y1, 2);
+    if (t == 0) {
+      ypart[cq * kGradRows + 16 * rg + g] = y0;
+      ypart[cq * kGradRows + 16 * rg + g + 8] = y1;
+    }
+    __syncthreads();
+    // ---- dz2 and the sums over rows that need no product
+    float dyn[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int r = 16 * rg + g + 8 * q;
+      const float yn = ypart[r] + ypart[kGradRows + r] + ypart[2 * kGradRows + r] +
+                       ypart[3 * kGradRows + r] + b3;
+      const float res = okr[r] != 0.f ? yn - tn[r] : 0.f;
+      dyn[q] = 2.f * res / (float)nrows;
+      if (cq == 0 && t == 0) {
+        l2 += res * res;
+        sdy += dyn[q];
+      }
+    }
+    // sums over the warp's 16 rows of its 32 columns (v[2 j + q]: column 8 j + 2 t + q),
+    // scattered over the row lanes: lane g ends with v[g], and adds it to the warp's
+    // own slot (shared-memory atomics on one address per column cost more than the MMAs)
+    auto colsum = [&](float *dst, float (&v)[8]) {
+#pragma unroll
+      for (int s = 4; s >= 1; s >>= 1) {
+        const bool up = g & s;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (k < s) {
+            const float keep = up ? v[k + s] : v[k], give = up ? v[k] : v[k + s];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * s);
+          }
+      }
+      dst[rg * W + 32 * cq + 8 * (g >> 1) + 2 * t + (g & 1)] += v[0];
+    };
+    float s3[8], s2[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 w = *reinterpret_cast<const float2 *>(w3 + 32 * cq + 8 * j + 2 * t);
+      s3[2 * j] = dyn[0] * c2[j][0] + dyn[1] * c2[j][2];
+      s3[2 * j + 1] = dyn[0] * c2[j][1] + dyn[1] * c2[j][3];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float h0 = c2[j][2 * q], h1v = c2[j][2 * q + 1];
+        c2[j][2 * q] = dyn[q] != 0.f ? dyn[q] * w.x * (1.f - h0 * h0) : 0.f;
+        c2[j][2 * q + 1] = dyn[q] != 0.f ? dyn[q] * w.y * (1.f - h1v * h1v) : 0.f;
+      }
+      s2[2 * j] = c2[j][0] + c2[j][2];
+      s2[2 * j + 1] = c2[j][1] + c2[j][3];
+      put(Ly::Z2, j, c2[j]);
+    }
+    colsum(gw3, s3);
+    colsum(gb2, s2);
+    __syncthreads();
+    // ---- dz1 = (dz2 W2)(1 - h1^2): B from W2 [j][k] by transposed loads
+    float z1[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) z1[j][0] = z1[j][1] = z1[j][2] = z1[j][3] = 0.f;
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk) {
+      uint32_t ah[4], al[4], r0[4], r1[4];
+      ldsm4(ah, a_at(sb + Ly::Z2, LD2, 16 * rg, kk));
+      ldsm4(al, a_at(sb + Ly::Z2 + 2 * kGradRows * LD2, LD2, 16 * rg, kk));
+      const uint32_t o = aW2 + 2u * (uint32_t)((16 * kk + bro) * LD2 + 32 * cq + bco);
+      ldsm4t(r0, o);
+      ldsm4t(r1, o + 32);
+      mma16816(z1[0], ah, r0[0], r0[1]);
+      mma16816(z1[1], ah, r0[2], r0[3]);
+      mma16816(z1[2], ah, r1[0], r1[1]);
+      mma16816(z1[3], ah, r1[2], r1[3]);
+      mma16816(z1[0], al, r0[0], r0[1]);
+      mma16816(z1[1], al, r0[2], r0[3]);
+      mma16816(z1[2], al, r1[0], r1[1]);
+      mma16816(z1[3], al, r1[2], r1[3]);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) z1[j][q] *= 1.f - h1[j][q] * h1[j][q];
+      s2[2 * j] = z1[j][0] + z1[j][2];
+      s2[2 * j + 1] = z1[j][1] + z1[j][3];
+      put(Ly::Z1, j, z1[j]);
+    }
+    colsum(gb1, s2);
+    __syncthreads();
+    // ---- dW2 += dz2^T h1 and dW1 += dz1^T xn, K = the tile's rows.  A tile's products
+    // start from zero and are added in FP32: the tensor core truncates its
+    // accumulator, which over hundreds of rows is a bias
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      float c[4][4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) c[j][0] = c[j][1] = c[j][2] = c[j][3] = 0.f;
+#pragma unroll
+      for (int kk = 0; kk < kGradRows / 16; ++kk) {
+        uint32_t ah[4], al[4];
+        uint32_t o = sb + Ly::Z2 + 2u * (uint32_t)((16 * kk + tro) * LD2 + 16 * jb + tco);
+        ldsm4t(ah, o);
+        ldsm4t(al, o + 2 * kGradRows * LD2);
+        o = sb + Ly::H1 + 2u * (uint32_t)((16 * kk + bro) * LD2 + 64 * kb + 32 * half + bco);
+#pragma unroll
+        for (int j = 0; j < 4; j += 2) {
+          uint32_t bh[4], bl[4];
+          ldsm4t(bh, o + 16 * j);
+          ldsm4t(bl, o + 16 * j + 2 * kGradRows * LD2);
+          mma16816(c[j], ah, bh[0], bh[1]);
+          mma16816(c[j + 1], ah, bh[2], bh[3]);
+          mma16816(c[j], ah, bl[0], bl[1]);
+          mma16816(c[j + 1], ah, bl[2], bl[3]);
+          mma16816(c[j], al, bh[0], bh[1]);
+          mma16816(c[j + 1], al, bh[2], bh[3]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) gW2[4 * half + j][q] += c[j][q];
+    }
+    {
+      float c[NT1][4];
+#pragma unroll
+      for (int j = 0; j < NT1; ++j) c[j][0] = c[j][1] = c[j][2] = c[j][3] = 0.f;
+#pragma unroll
+      for (int kk = 0; kk < kGradRows / 16; ++kk) {
+        uint32_t ah[4], al[4];
+        uint32_t o = sb + Ly::Z1 + 2u * (uint32_t)((16 * kk + tro) * LD2 + 16 * jb + tco);
+        ldsm4t(ah, o);
+        ldsm4t(al, o + 2 * kGradRows * LD2);
+        o = sb + Ly::X + 2u * (uint32_t)((16 * kk + (lane & 15)) * LD1 + 8 * NT1 * kb);
+#pragma unroll
+        for (int j = 0; j < NT1; ++j) {
+          uint32_t bh[2], bl[2];
+          ldsm2t(bh, o + 16 * j);
+          ldsm2t(bl, o + 16 * j + 2 * kGradRows * LD1);
+          mma16816(c[j], ah, bh[0], bh[1]);
+          mma16816(c[j], ah, bl[0], bl[1]);
+          mma16816(c[j], al, bh[0], bh[1]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < NT1; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) gW1[j][q] += c[j][q];
+    }
+  }
+  // the CTA's partial gradient, in the order of the parameters, made in shared memory
+  // (over the tile's buffers) and written by one bulk copy
+  for (int o = 16; o > 0; o >>= 1) {
+    l2 += __shfl_xor_sync(0xffffffffu, l2, o);
+    sdy += __shfl_xor_sync(0xffffffffu, sdy, o);
+  }
+  if (cq == 0 && lane == 0) {
+    if (loss) atomicAdd(loss, l2 / (float)nrows);
+    atomicAdd(gb3, sdy);
+  }
+  __syncthreads();
+  float *P = reinterpret_cast<float *>(sm + Ly::X), *P2 = P + W * d + W;  // P2: 16-byte aligned
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int k = 64 * kb + 8 * j + 2 * t;
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      *reinterpret_cast<float2 *>(P2 + (16 * jb + g + 8 * q) * W + k) =
+          make_float2(gW2[j][2 * q], gW2[j][2 * q + 1]);
+  }
+#pragma unroll
+  for (int j = 0; j < NT1; ++j) {
+    const int k = 8 * (NT1 * kb + j) + 2 * t;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (k + (q & 1) < d) P[(16 * jb + g + 8 * (q >> 1)) * d + k + (q & 1)] = gW1[j][q];
+  }
+  if (tid < W) {
+    auto sum4 = [&](const float *v) { return (v[tid] + v[W + tid]) + (v[2 * W + tid] + v[3 * W + tid]); };
+    P[W * d + tid] = sum4(gb1);
+    P2[W * W + tid] = sum4(gb2);
+    P2[W * W + W + tid] = sum4(gw3);
+  }
+  if (tid < 4) P2[W * W + 2 * W + tid] = tid == 0 ? *gb3 : 0.f;  // and the padding
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncthreads();
+  if (tid == 0) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                     part + (long long)blockIdx.x * part_stride(d)),
+                 "r"(sb + Ly::X), "r"(part_stride(d) * 4)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // shared memory is read
+  }
+}
+
+// g = sum of the partial gradients; with adam, the update of k_mlp_adam on top (g is
+// then left zero, as that kernel leaves it).  64 parameters per CTA, the partials in
+// four interleaved groups.
+__global__ void __launch_bounds__(256) k_mlp_tc_reduce(MlpDev M, int np, int nparts,
+                                                       const float *__restrict__ part, int adam,
+                                                       float lr, float b1, float b2, float eps,
+                                                       int step, int k1,
+                                                       unsigned char *__restrict__ im) {
+  __shared__ float sh[4][64];
+  const int c = threadIdx.x & 63, grp = threadIdx.x >> 6, q = blockIdx.x * 64 + c;
+  float s = 0.f;
+  if (q < np) {
+#pragma unroll 8
+    for (int k = grp; k < nparts; k += 4) s += part[(long long)k * part_stride(M.d) + q];
+  }
+  sh[grp][c] = s;
+  __syncthreads();
+  if (grp || q >= np) return;
+  const float g = (sh[0][c] + sh[1][c]) + (sh[2][c] + sh[3][c]);
+  if (!adam) {
+    M.g[q] = g;
+    return;
+  }
+  const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
+  const float m = b1 * M.m[q] + (1.f - b1) * g;
+  const float v = b2 * M.v[q] + (1.f - b2) * g * g;
+  M.m[q] = m;
+  M.v[q] = v;
+  const float w = M.p[q] - lr * (m / c1) / (sqrtf(v / c2) + eps);
+  M.p[q] = w;
+  image_put(im, M.d, k1, q, w);  // for the next step
 }
 
 template <int K1>
@@ -676,30 +770,19 @@ cudaError_t infer_k(const MlpDev &M, const float *x, int n, float *y, cudaStream
 }
 
 template <int K1>
-cudaError_t wgrad_k(const MlpDev &M, int nrows, const float *store, const float *bw,
-                    cudaStream_t s) {
-  cudaError_t e = smem_optin_once<k_mlp_tc_wgrad<K1>>();
+cudaError_t grad_k(const MlpDev &M, const float *x, const float *t, int n, int nrows, int sampled,
+                   uint64_t seed, int step, const unsigned char *im, float *part, int nparts,
+                   float *loss, cudaStream_t s) {
+  cudaError_t e = smem_optin_once<k_mlp_tc_grad<K1>>();
   if (e != cudaSuccess) return e;
-  dim3 grid((nrows + kRowsPerCta - 1) / kRowsPerCta, 2);
-  k_mlp_tc_wgrad<K1><<<grid, kThreads, wgrad_smem_tc(), s>>>(M, nrows, store, bw);
+  k_mlp_tc_grad<K1><<<nparts, kGradThreads, GradLay<K1>::bytes, s>>>(
+      M, x, t, n, nrows, sampled, seed, step, im, part, loss);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 bool mlp_tc_supported(int d, int w) { return w == W && d >= 1 && d <= 64; }
-
-cudaError_t mlp_tc_forward(const MlpDev &M, const float *x, int n, const int *idx, int nrows,
-                           float *y, float *store, cudaStream_t s) {
-  if (nrows <= 0) return cudaSuccess;
-  const int k1 = (M.d + 15) / 16 * 16;
-  switch (k1) {
-    case 16: return forward_k<16>(M, x, n, idx, nrows, y, store, s);
-    case 32: return forward_k<32>(M, x, n, idx, nrows, y, store, s);
-    case 48: return forward_k<48>(M, x, n, idx, nrows, y, store, s);
-    default: return forward_k<64>(M, x, n, idx, nrows, y, store, s);
-  }
-}
 
 cudaError_t mlp_tc_infer(const MlpDev &M, const float *x, int n, float *y, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
@@ -711,26 +794,36 @@ cudaError_t mlp_tc_infer(const MlpDev &M, const float *x, int n, float *y, cudaS
   }
 }
 
-cudaError_t mlp_tc_backward_rows(const MlpDev &M, const float *t, const int *idx, int nrows,
-                                 const float *store, float *bw, float *loss, cudaStream_t s) {
-  if (nrows <= 0) return cudaSuccess;
-  cudaError_t e = smem_optin_once<k_mlp_tc_backward_rows>();
-  if (e != cudaSuccess) return e;
-  k_mlp_tc_backward_rows<<<(nrows + kRowsPerCta - 1) / kRowsPerCta, kThreads, bwd_smem_tc(), s>>>(
-      M, t, idx, nrows, store, bw, loss);
+size_t mlp_tc_image_bytes(int d) { return image_bytes((d + 15) / 16 * 16); }
+
+cudaError_t mlp_tc_image(const MlpDev &M, unsigned char *im, cudaStream_t s) {
+  const int np = M.w * M.d + M.w + M.w * M.w + M.w + M.w + 1;
+  k_mlp_tc_image<<<(np + 255) / 256, 256, 0, s>>>(M, (M.d + 15) / 16 * 16, np, im);
   return cudaGetLastError();
 }
 
-cudaError_t mlp_tc_wgrad(const MlpDev &M, int nrows, const float *store, const float *bw,
-                         cudaStream_t s) {
-  if (nrows <= 0) return cudaSuccess;
-  const int k1 = (M.d + 15) / 16 * 16;
-  switch (k1) {
-    case 16: return wgrad_k<16>(M, nrows, store, bw, s);
-    case 32: return wgrad_k<32>(M, nrows, store, bw, s);
-    case 48: return wgrad_k<48>(M, nrows, store, bw, s);
-    default: return wgrad_k<64>(M, nrows, store, bw, s);
+size_t mlp_tc_part_bytes(int d) { return (size_t)part_stride(d) * sizeof(float); }
+
+int mlp_tc_parts(int nrows) { return std::min((nrows - 1) / kGradRows + 1, 152); }
+
+cudaError_t mlp_tc_grad(const MlpDev &M, const float *x, const float *t, int n, int nrows, int sampled,
+                        uint64_t seed, int step, const unsigned char *im, float *part, float *loss,
+                        cudaStream_t s) {
+  const int np = mlp_tc_parts(nrows);
+  switch ((M.d + 15) / 16 * 16) {
+    case 16: return grad_k<16>(M, x, t, n, nrows, sampled, seed, step, im, part, np, loss, s);
+    case 32: return grad_k<32>(M, x, t, n, nrows, sampled, seed, step, im, part, np, loss, s);
+    case 48: return grad_k<48>(M, x, t, n, nrows, sampled, seed, step, im, part, np, loss, s);
+    default: return grad_k<64>(M, x, t, n, nrows, sampled, seed, step, im, part, np, loss, s);
   }
+}
+
+cudaError_t mlp_tc_reduce(const MlpDev &M, int nparts, const float *part, int adam, float lr, float b1,
+                          float b2, float eps, int step, unsigned char *im, cudaStream_t s) {
+  const int np = M.w * M.d + M.w + M.w * M.w + M.w + M.w + 1;
+  k_mlp_tc_reduce<<<(np + 63) / 64, 256, 0, s>>>(M, np, nparts, part, adam, lr, b1, b2, eps, step,
+                                                 (M.d + 15) / 16 * 16, im);
+  return cudaGetLastError();
 }
 
 }  // namespace bsi

@@ -225,3 +225,62 @@ def test_surrogate_error_bars_on_held_out_masks():
     plan.close()
     assert max(err_net) <= 0.10
     assert np.mean(err_net) < np.mean(err_16)
+
+
+@pytest.mark.parametrize("d", [1, 16, 45, 64])
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 127, 128, 129, 152 * 64 + 65])
+def test_tensor_kernels_at_ragged_rows(n, d):
+    """Rows around the 64-row tile of the gradient and the 128-row tile of the
+    forward pass, one row, and more tiles than blocks; the smallest, a whole,
+    an odd and the largest input width; rows that start off a 16-byte boundary.
+    The network's output is good to e = 1e-4 of its scale, as in
+    test_forward_and_gradient_match_fp64_reference; residuals r carry that error
+    into the loss (2 e |r| + e^2) and the gradient (e / |r| of it)."""
+    torch = _torch()
+    import paper_2506_10526_gb300 as bs
+    r = np.random.default_rng(100 * d + n)
+    x = (r.standard_normal((n + 1, d)) * 2 + 0.5).astype(np.float32)
+    t = r.standard_normal(n + 1).astype(np.float32)
+    net = bs.Surrogate(d, 128, seed=7)
+    net.set_kernels("tensor")
+    xd, td = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+    net.fit_norm(xd, td)
+    p = net.params().astype(np.float64)
+    nw = net.n_weights
+    norm = (p[nw:nw + d], p[nw + d:nw + 2 * d], p[nw + 2 * d], p[nw + 2 * d + 1])
+    xs, ts = x[1:].astype(np.float64), t[1:].astype(np.float64)
+    y = net.forward(xd[1:]).cpu().numpy()
+    y_ref, _ = omlp.forward(p[:nw], xs, d, 128, norm, bf16=True)
+    yn, tn = (y_ref - norm[2]) / norm[3], (ts - norm[2]) / norm[3]
+    e, res = 1e-4 * max(1.0, np.abs(yn).max()), np.sqrt(np.mean((yn - tn) ** 2))
+    assert np.all(np.abs(y - y_ref) <= e * norm[3] + 1e-6 * abs(norm[2]))
+    loss, g = net.grad(xd[1:], td[1:])
+    loss_ref, g_ref = omlp.loss_and_grad(p[:nw], xs, ts, d, 128, norm, bf16=True)
+    tol_loss = 2 * e * res + e * e
+    assert abs(loss - loss_ref) <= tol_loss
+    np.testing.assert_allclose(g, g_ref, rtol=0, atol=(2e-4 + e / res) * np.abs(g_ref).max())
+    if n == 1:  # one training step over 65 draws of the only row: that row's loss
+        loss = net.train(xd[1:], td[1:], steps=1, batch=65, lr=1e-3)
+        assert abs(loss - loss_ref) <= tol_loss
+    net.close()
+
+
+@pytest.mark.parametrize("n", [2, 63, 64, 65, 152 * 64 + 1])
+@pytest.mark.parametrize("d", [1, 31, 32, 45, 64])
+def test_column_statistics(n, d):
+    """Mean and standard deviation of every column: fewer and more rows than
+    warps, columns around a warp's 32 lanes.  FP64 sums, rounded once to FP32
+    (2^-24 = 6e-8); the mean is zero to 6e-8 of the spread."""
+    torch = _torch()
+    import paper_2506_10526_gb300 as bs
+    r = np.random.default_rng(n + d)
+    x = (r.standard_normal((n, d)) * 3 + 1).astype(np.float32)
+    t = r.standard_normal(n).astype(np.float32)
+    net = bs.Surrogate(d, 128, seed=1)
+    net.fit_norm(torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda())
+    got = net.params().astype(np.float64)[net.n_weights:]
+    net.close()
+    cols = np.concatenate([x, t[:, None]], axis=1).astype(np.float64)
+    mean, sd = cols.mean(0), cols.std(0)
+    want = np.concatenate([mean[:d], sd[:d], mean[d:], sd[d:]])
+    np.testing.assert_allclose(got, want, rtol=1e-7, atol=1e-7)
