@@ -464,3 +464,35 @@ def test_contraction_forms_over_ragged_blocks(block, precision):
                     np.add.at(size, at, babs[t][n1, n2, n3] * scale)
                 assert np.all(np.abs(got[t] - want) <= TOL[precision] * size)
         plan.close()
+
+
+@pytest.mark.parametrize("cmax,side", [(5, 16), (7, 24), (10, 32), (15, 48), (21, 64), (31, 96),
+                                       (42, 128), (63, 192), (85, 256), (127, 384), (170, 512),
+                                       (255, 768)])
+def test_every_register_transform_side(cmax, side):
+    """Each image side with a register transform, three channels of two
+    realisations (row pairs that fill the last block of rows to a part only),
+    FP32 rows and split BF16 rows: triples of an inner and an outermost ring
+    against the oracle."""
+    torch = _torch()
+    import paper_2506_10526_gb300 as bs
+    nt, nc, edges = 2 * cmax + 2, 3, [1.0, 2.3, cmax - 0.6, cmax + 0.2]
+    vis = np.stack([synth.sky_visibilities(nt, nc, seed=side + k) for k in range(2)])
+    trips = [(0, 0, 0), (0, 2, 2), (2, 2, 2)]
+    refs = [(oracle.mabs_full(v, edges, triples=trips),
+             oracle.mabs_full(np.abs(v), edges, triples=trips)) for v in vis]
+    for precision in (0, 1):
+        plan = bs.Plan(nt, nc, edges, precision=precision, batch=2)
+        assert plan.M == side
+        index = [oracle.ring_triples(3).index(t) for t in trips]
+        plan.grid_load(torch.from_numpy(vis.astype(np.complex64)).cuda())
+        full = torch.empty((2, plan.ntrip, nc, nc, nc), dtype=torch.float64, device="cuda")
+        plan.mabs(out_full=full)
+        torch.cuda.synchronize()
+        got = full.cpu().numpy()[:, index]
+        plan.close()
+        for k, (ref, mag) in enumerate(refs):
+            want, size = ref["B"].real, mag["B"].real
+            ok = ~np.isnan(want)
+            assert np.array_equal(np.isnan(got[k]), ~ok)
+            assert np.all(np.abs(got[k][ok] - want[ok]) <= TOL[precision] * size[ok])
