@@ -34,8 +34,8 @@ namespace {
 // deviations, NaN values skipped.  CH values at a time: their own mean and sum of
 // squared deviations (3 FP64 operations a value), merged into the running ones by
 // the pairwise update of Chan, Golub & LeVeque (one division per CH values).  FP64
-// issue bounds the kernel, not HBM; Welford's update, which CH = 1 keeps for fewer
-// than four realisations, takes a division for every value (256 realisations of the
+// issue bounds the kernel, not HBM; Welford's update, which CH = 1 keeps for one
+// realisation, takes a division for every value (256 realisations of the
 // 64^2 x 16 channel grid: 0.63 ms per call of the 3D bispectrum and the collapse).
 __device__ __forceinline__ bool is_nan_bits(double v) {
   const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
@@ -72,7 +72,7 @@ __global__ void k_welford(const double *__restrict__ x, int batch, long long n, 
             ++k;
           }
         if (k == 0) continue;
-        const double kd = (double)k, mb = sum / kd;
+        const double kd = (double)k, mb = k == CH ? sum * (1.0 / CH) : sum / kd;  // exact: CH = 2^n
 #pragma unroll
         for (int u = 0; u < CH; ++u)
           if (!is_nan_bits(v[u])) {
@@ -95,6 +95,8 @@ void launch_welford(const double *x, int batch, long long n, double *st, cudaStr
   const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
   if (batch >= 16)
     k_welford<16><<<blocks, 256, 0, s>>>(x, batch, n, st, st + n, st + 2 * n);
+  else if (batch >= 2 && batch < 4)
+    k_welford<2><<<blocks, 256, 0, s>>>(x, batch, n, st, st + n, st + 2 * n);
   else if (batch >= 4)
     k_welford<4><<<blocks, 256, 0, s>>>(x, batch, n, st, st + n, st + 2 * n);
   else

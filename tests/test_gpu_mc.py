@@ -287,3 +287,56 @@ def test_mc_channel_symmetric_cubes_match_the_plan(precision):
             assert np.array_equal(np.isnan(got), np.isnan(want)), g
             for k in range(want.shape[0]):
                 assert np.all(np.abs(got[k] - want[k])[ok[k]] <= beta[k]), (g, k)
+
+
+@pytest.mark.parametrize("batch", [1, 2, 3, 4, 5, 16, 17])
+def test_statistics_of_every_batch_form(batch):
+    """Realisations per pass around the groups the statistics take at a time (1, 2,
+    4 and 16), two passes: mean and variance against numpy over the realisations
+    taken one by one (a pass of one realisation has that value as its mean).  A
+    value's contraction may differ by FP32 summation order between the two batch
+    sizes: 1e-4 of the largest value, far above it and far below a missing or
+    doubled realisation."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2506_10526_gb300 as bs
+    spec = dict(nt=24, nchan=6, edges=list(synth.edges_linear(4, 12)))
+    flags = np.zeros(6, np.uint8)
+    flags[[0, 1]] = 1  # unsampled delays: NaN bins
+    x = np.stack([synth.sky_visibilities(24, 6, 4000 + k) for k in range(2 * batch)])
+    x = torch.from_numpy(x.astype(np.complex64)).cuda()
+
+    def ensemble(b):
+        ens = bs.Ensemble([dict(spec, batch=b)])
+        buf = torch.empty((b, 6, 24, 24), dtype=torch.complex64, device="cuda")
+        ens.set_input(0, buf)
+        ens.set_flags(0, flags)
+        return ens, buf
+
+    ens, buf = ensemble(batch)
+    for r in range(2):
+        buf.copy_(x[r * batch:(r + 1) * batch])
+        ens.run()
+    got = [ens.stats(0, w) for w in (0, 1)]
+    ens.close()
+    ens, buf = ensemble(1)
+    single = []
+    for r in range(2 * batch):
+        ens.reset()
+        buf.copy_(x[r:r + 1])
+        ens.run()
+        single.append([ens.stats(0, w)[0] for w in (0, 1)])
+    ens.close()
+    for which in (0, 1):
+        ref = np.array([s[which] for s in single])
+        mean, var, n = got[which]
+        assert n == 2 * batch
+        bad = np.isnan(ref[0])
+        assert bad.any() or which == 1
+        assert np.array_equal(np.isnan(mean), bad)
+        ok = ~bad
+        tol = 1e-4 * np.abs(ref[:, ok]).max()
+        want_v = ref[:, ok].var(axis=0, ddof=1)
+        assert np.all(np.abs(mean[ok] - ref[:, ok].mean(axis=0)) <= tol)
+        assert np.all(np.abs(var[ok] - want_v) <= 2 * np.sqrt(want_v) * tol + tol ** 2)
