@@ -25,9 +25,9 @@
 // The kernel it replaced transposed every 16-pixel chunk through scalar stores
 // with 4-way bank conflicts, kept the pair operand in shared memory and stopped at
 // three barriers per chunk.  32 channels, 256^2 grid, 20 rings, ten image sides:
-// 29.8 ms, 121.4 before (1.45e12 FLOP: 49 and 12 TFLOP/s of the 76.6 measured; the
+// 28.4 ms, 121.4 before (1.45e12 FLOP: 51 and 12 TFLOP/s of the 76.6 measured; the
 // rest is padding of the tiles); 27 channels, 90^2 grid, 7 rings, two
-// realisations: 4.2 ms, 9.3 before.
+// realisations: 4.0 ms, 9.3 before.
 //
 // Partial sums are FP32, folded into a second FP32 set (in shared memory) every
 // 1024 pixels: two-level summation bounds the rounding growth over long K.  The
@@ -82,6 +82,10 @@ __device__ __forceinline__ void simt_tile(const ContractArgs &a, const SimtTile 
                                           float *sm, ColInfo &ci) {
   constexpr int NCOL = 128 / H, TX = NCOL / 8, NR = TR1 + TR2 * H + NCOL;
   constexpr int STAGE = NR * PITCH, NCP = (NR * (KC / 4) + kSimtThreads - 1) / kSimtThreads;
+  // column of staged row r: a thread's columns are runs of four (c & 3 = its step), so
+  // the reduction below adds an entry's terms by c & 3 within a row of the pair
+  // rectangle, whatever H; staged so that a load's 8 rows are adjacent
+  auto col_of = [](int r) { return 4 * (r % TX) + (r / TX & 3) + 4 * TX * (r / TX >> 2); };
   const int tid = threadIdx.x;
   const int n_r1 = (a.nu1_hi - a.nu1_lo + TR1 - 1) / TR1;
   const int n_r2 = (a.nu2_hi - a.nu2_lo + TR2 * H - 1) / (TR2 * H);
@@ -150,7 +154,7 @@ __device__ __forceinline__ void simt_tile(const ContractArgs &a, const SimtTile 
       const int nu2 = nu2_0 + r - TR1;
       if (nu2 < a.nu2_hi) f = (long long)pt.rj * a.nc + nu2;
     } else if (r < NR) {
-      f = ci.field[r - TR1 - TR2 * H];
+      f = ci.field[col_of(r - TR1 - TR2 * H)];
     }
     have[m] = f >= 0;
     src[m] = Fb + (f >= 0 ? f * lv.M2 : 0) + 4 * (q & 7);
@@ -254,8 +258,9 @@ __device__ __forceinline__ void simt_tile(const ContractArgs &a, const SimtTile 
     const int nu1 = nu1_0 + i0 + 8 * (y >> 2), nu2 = nu2_0 + j0 + (y & 3);
     if (nu1 >= a.nu1_hi || nu2 >= a.nu2_hi) continue;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int c = tx + TX * u;
+    for (int step = 0; step < 8; ++step) {
+      const int u = H == 1 ? step : (step >> 1) + 4 * (step & 1);
+      const int c = col_of(tx + TX * u);
       if (ci.field[c] < 0) continue;
       const uint64_t v = acc[(y >> 2) * 2 + ((y & 3) >> 1)][u];
       const float s = (y & 1) ? hi_f(v) : lo_f(v);
