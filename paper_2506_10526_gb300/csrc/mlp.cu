@@ -32,7 +32,7 @@ using namespace bsi;
 namespace {
 
 constexpr int kMaxD = 64, kMaxW = 128, kRows = 128;
-constexpr int kStatParts = 152;  // CTAs of the column statistics
+constexpr int kStatParts = 152, kStatThreads = 1024;  // CTAs of the column statistics, threads each
 
 __device__ __forceinline__ float bf(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
@@ -212,9 +212,10 @@ __global__ void k_mlp_sample(int *idx, int nrows, int n, unsigned long long seed
 
 // Column means and standard deviations (FP64 sums) of x [n][d] and t [n].  A warp walks
 // whole rows, lane = column (and column + 32, + 64..): coalesced reads.  One CTA per
-// column read a float every d: 244 us for 122880 x 45, 70 for both kernels here.  Each CTA leaves its sums in
+// column read a float every d: 244 us for 122880 x 45; with both kernels here 70 us
+// at 8 warps a CTA, 49 at 32 (more rows in flight).  Each CTA leaves its sums in
 // sums[CTA][2][d + 1]; k_mlp_norm adds them up.
-__global__ void __launch_bounds__(256) k_mlp_colstats(const float *__restrict__ x,
+__global__ void __launch_bounds__(kStatThreads) k_mlp_colstats(const float *__restrict__ x,
                                                       const float *__restrict__ t, int n, int d,
                                                       double *__restrict__ sums) {
   __shared__ double sh[2][kMaxD + 1];
@@ -521,7 +522,7 @@ bs_status bs_mlp_fit_norm(bs_mlp m, const float *x_dev, const float *t_dev, int 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int d = m->dev.d;
   const int parts = std::min(kStatParts, (n + 63) / 64);
-  k_mlp_colstats<<<parts, 256, 0, s>>>(x_dev, t_dev, n, d, m->stat);
+  k_mlp_colstats<<<parts, kStatThreads, 0, s>>>(x_dev, t_dev, n, d, m->stat);
   ML_CUDA(cudaGetLastError());
   k_mlp_norm<<<1, 1024, 0, s>>>(m->stat, parts, n, d, m->dev.norm);
   ML_CUDA(cudaGetLastError());
