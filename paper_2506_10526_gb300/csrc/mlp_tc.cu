@@ -153,6 +153,28 @@ __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
                : "r"(addr));
 }
 
+// Programmatic dependent launch.  A training step is two kernels of 4 and 16 us: the
+// next one's blocks start while the last blocks of this one run (pdl_launch, once all
+// have started), and wait (pdl_wait: complete and visible) before they touch what it
+// writes.  The gradient kernel has its first rows staged by then.  24 steps with one
+// large gradient and the statistics: 1.00 ms, 0.88 with it.
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
 // B fragments of n-tiles j, j + 1 (rows 8j .. 8j + 15 of a weight matrix stored
 // [n][k]) at k-step kk: the address this lane gives to ldsm4; r[0], r[1] are tile
 // j's two registers, r[2], r[3] tile j + 1's.
@@ -401,17 +423,14 @@ __global__ void __launch_bounds__(kGradThreads, 1)
   const int jb = warp & 7, kb = warp >> 3;   // weight gradients: rows 16 jb.., half kb of the inputs
   const uint32_t sb = (uint32_t)__cvta_generic_to_shared(sm);
   const uint32_t aW1 = sb + Ly::W1s, aW2 = sb + Ly::W2s;
-  for (int q = tid; q < (Ly::net + 3 * W * 4) / 16; q += kGradThreads)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sb + 16u * q), "l"(im + 16 * q)
-                 : "memory");
-  asm volatile("cp.async.commit_group;" ::: "memory");
+  pdl_launch();
   for (int q = tid; q < 12 * W; q += kGradThreads) gb1[q] = 0.f;
   if (tid == 0) *gb3 = 0.f;
   for (int k = tid; k < K1; k += kGradThreads) {
     mu[k] = k < d ? M.norm[k] : 0.f;
     inv[k] = k < d ? 1.f / M.norm[d + k] : 0.f;
   }
-  const float b3 = M.p[(long long)W * d + W + W * W + W + W];
+  float b3 = 0.f;
   const float my = M.norm[2 * d], sy = M.norm[2 * d + 1];
   float l2 = 0.f, sdy = 0.f;  // sums of squared residuals and of dyn
   float gW2[8][4], gW1[NT1][4];
@@ -453,7 +472,14 @@ __global__ void __launch_bounds__(kGradThreads, 1)
       *reinterpret_cast<uint32_t *>(sm + Ly::X + 2 * (r * LD1 + c)) = hi;
       *reinterpret_cast<uint32_t *>(sm + Ly::X + 2 * (kGradRows * LD1 + r * LD1 + c)) = lo;
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");  // the network (first tile)
+    if (tile == (int)blockIdx.x) {  // the network, once the previous step has updated it
+      pdl_wait();
+      for (int q = tid; q < (Ly::net + 3 * W * 4) / 16; q += kGradThreads)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sb + 16u * q), "l"(im + 16 * q)
+                     : "memory");
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      b3 = M.p[(long long)W * d + W + W * W + W + W];
+    }
     __syncthreads();
     // ---- forward 1
     float h1[4][4];
@@ -736,6 +762,8 @@ __global__ void __launch_bounds__(256) k_mlp_tc_reduce(MlpDev M, int np, int npa
   __shared__ float sh[4][64];
   const int c = threadIdx.x & 63, grp = threadIdx.x >> 6, q = blockIdx.x * 64 + c;
   float s = 0.f;
+  pdl_launch();
+  pdl_wait();
   if (q < np) {
 #pragma unroll 8
     for (int k = grp; k < nparts; k += 4) s += part[(long long)k * part_stride(M.d) + q];
@@ -775,9 +803,8 @@ cudaError_t grad_k(const MlpDev &M, const float *x, const float *t, int n, int n
                    float *loss, cudaStream_t s) {
   cudaError_t e = smem_optin_once<k_mlp_tc_grad<K1>>();
   if (e != cudaSuccess) return e;
-  k_mlp_tc_grad<K1><<<nparts, kGradThreads, GradLay<K1>::bytes, s>>>(
-      M, x, t, n, nrows, sampled, seed, step, im, part, loss);
-  return cudaGetLastError();
+  return launch_pdl(k_mlp_tc_grad<K1>, nparts, kGradThreads, GradLay<K1>::bytes, s, M, x, t, n, nrows,
+                    sampled, (unsigned long long)seed, step, im, part, loss);
 }
 
 }  // namespace
@@ -821,9 +848,8 @@ cudaError_t mlp_tc_grad(const MlpDev &M, const float *x, const float *t, int n, 
 cudaError_t mlp_tc_reduce(const MlpDev &M, int nparts, const float *part, int adam, float lr, float b1,
                           float b2, float eps, int step, unsigned char *im, cudaStream_t s) {
   const int np = M.w * M.d + M.w + M.w * M.w + M.w + M.w + 1;
-  k_mlp_tc_reduce<<<(np + 63) / 64, 256, 0, s>>>(M, np, nparts, part, adam, lr, b1, b2, eps, step,
-                                                 (M.d + 15) / 16 * 16, im);
-  return cudaGetLastError();
+  return launch_pdl(k_mlp_tc_reduce, (np + 63) / 64, 256, 0, s, M, np, nparts, part, adam, lr, b1, b2,
+                    eps, step, (M.d + 15) / 16 * 16, im);
 }
 
 }  // namespace bsi
