@@ -406,7 +406,7 @@ template <int K1>
 __global__ void __launch_bounds__(kGradThreads, 1)
     k_mlp_tc_grad(MlpDev M, const float *__restrict__ x, const float *__restrict__ tgt, int n,
                   int nrows, int sampled, unsigned long long seed, int step,
-                  const unsigned char *__restrict__ im, float *__restrict__ part,
+                  const unsigned char *im, float *__restrict__ part,
                   float *__restrict__ loss) {
   using Ly = GradLay<K1>;
   constexpr int LD1 = K1 + 8, KS1 = K1 / 16, NT1 = K1 / 16;  // dW1 n-tiles of a warp
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(kGradThreads, 1)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sb + 16u * q), "l"(im + 16 * q)
                      : "memory");
       asm volatile("cp.async.wait_all;" ::: "memory");
-      b3 = M.p[(long long)W * d + W + W * W + W + W];
+      b3 = __ldcg(M.p + (long long)W * d + W + W * W + W + W);  // the step before writes it
     }
     __syncthreads();
     // ---- forward 1
@@ -751,11 +751,15 @@ __global__ void __launch_bounds__(kGradThreads, 1)
   }
 }
 
-// g = sum of the partial gradients; with adam, the update of k_mlp_adam on top (g is
-// then left zero, as that kernel leaves it).  64 parameters per CTA, the partials in
-// four interleaved groups.
+// g = sum of the partial gradients; with adam, the update of k_mlp_adam on top instead
+// (M.g is not touched).  64 parameters per CTA, the partials in four interleaved groups.
+//
+// The blocks are resident while the gradient kernel still writes `part` (pdl_launch), so
+// the partials change during this kernel's life: they are read after pdl_wait through L2
+// (__ldcg), never through the read-only path that a __restrict__ pointer to constant
+// data allows.
 __global__ void __launch_bounds__(256) k_mlp_tc_reduce(MlpDev M, int np, int nparts,
-                                                       const float *__restrict__ part, int adam,
+                                                       const float *part, int adam,
                                                        float lr, float b1, float b2, float eps,
                                                        int step, int k1,
                                                        unsigned char *__restrict__ im) {
@@ -766,7 +770,7 @@ __global__ void __launch_bounds__(256) k_mlp_tc_reduce(MlpDev M, int np, int npa
   pdl_wait();
   if (q < np) {
 #pragma unroll 8
-    for (int k = grp; k < nparts; k += 4) s += part[(long long)k * part_stride(M.d) + q];
+    for (int k = grp; k < nparts; k += 4) s += __ldcg(part + (long long)k * part_stride(M.d) + q);
   }
   sh[grp][c] = s;
   __syncthreads();

@@ -284,3 +284,28 @@ def test_column_statistics(n, d):
     mean, sd = cols.mean(0), cols.std(0)
     want = np.concatenate([mean[:d], sd[:d], mean[d:], sd[d:]])
     np.testing.assert_allclose(got, want, rtol=1e-7, atol=1e-7)
+
+
+@pytest.mark.parametrize("batch", [8192, 152 * 64 + 65])
+def test_consecutive_training_steps_see_each_other(batch):
+    """The kernels of consecutive steps overlap (dependent launch): forty steps of
+    one call against forty calls of one step, which draw the same rows, with fewer
+    and more 64-row tiles than SMs.  Runs differ by the order of FP32 sums only;
+    a partial gradient or a weight of an older step would move a parameter by the
+    order of the step, 1e-3.  Bound: a hundredth of one step."""
+    torch = _torch()
+    import paper_2506_10526_gb300 as bs
+    d, steps, lr = 45, 40, 1e-3
+    g = torch.Generator().manual_seed(5)
+    x = torch.randn((20000, d), generator=g).cuda()
+    t = (torch.tanh(x[:, 0].cpu()) + 0.5 * x[:, 1].cpu()).cuda()
+    out = []
+    for calls in ([steps], [1] * steps):
+        net = bs.Surrogate(d, 128, seed=3)
+        net.set_kernels("tensor")
+        net.fit_norm(x, t)
+        for k in calls:
+            net.train(x, t, steps=k, batch=batch, lr=lr, seed=11)
+        out.append(net.params())
+        net.close()
+    assert np.abs(out[0] - out[1]).max() <= 1e-2 * lr
