@@ -226,8 +226,8 @@ __global__ void __launch_bounds__(kStatThreads) k_mlp_colstats(const float *__re
   for (int c = lane; c <= d; c += 32) {
     double s = 0, s2 = 0;
 #pragma unroll 8
-    for (int r = w; r < n; r += nw) {
-      const double v = fpb::f32_to_f64_pow2(c < d ? x[(long long)r * d + c] : t[r], 0);
+    for (long long r = w; r < n; r += nw) {  // n may be any positive int: r + nw passes 2^31
+      const double v = fpb::f32_to_f64_pow2(c < d ? x[r * d + c] : t[r], 0);
       s += v;
       s2 = fma(v, v, s2);
     }
@@ -521,7 +521,7 @@ bs_status bs_mlp_fit_norm(bs_mlp m, const float *x_dev, const float *t_dev, int 
   if (!m || !x_dev || !t_dev || n < 2) return BS_ERR_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int d = m->dev.d;
-  const int parts = std::min(kStatParts, (n + 63) / 64);
+  const int parts = std::min(kStatParts, (n - 1) / 64 + 1);
   k_mlp_colstats<<<parts, kStatThreads, 0, s>>>(x_dev, t_dev, n, d, m->stat);
   ML_CUDA(cudaGetLastError());
   k_mlp_norm<<<1, 1024, 0, s>>>(m->stat, parts, n, d, m->dev.norm);

@@ -309,3 +309,25 @@ def test_consecutive_training_steps_see_each_other(batch):
         out.append(net.params())
         net.close()
     assert np.abs(out[0] - out[1]).max() <= 1e-2 * lr
+
+
+def test_column_statistics_of_the_largest_row_counts():
+    """A row count within one stride (152 blocks of 32 warps) of 2^31: the row
+    index of the walk passes the range of int.  Ones, with a thousand in the last
+    4000 rows, so that a row left out or taken twice moves the mean."""
+    torch = _torch()
+    import paper_2506_10526_gb300 as bs
+    n = 2 ** 31 - 1000
+    if torch.cuda.mem_get_info()[0] < 24 << 30:
+        pytest.skip("needs 24 GB of device memory")
+    x = torch.ones((n, 1), dtype=torch.float32, device="cuda")
+    t = torch.ones(n, dtype=torch.float32, device="cuda")
+    x[-4000:] = 1000.0
+    t[-4000:] = 1000.0
+    net = bs.Surrogate(1, 128, seed=1)
+    net.fit_norm(x, t)
+    got = net.params().astype(np.float64)[net.n_weights:]
+    net.close()
+    f = 4000.0 / n
+    mean, sd = 1.0 + 999.0 * f, 999.0 * np.sqrt(f * (1.0 - f))
+    np.testing.assert_allclose(got, [mean, sd, mean, sd], rtol=2e-7)
