@@ -30,11 +30,14 @@
 #include <algorithm>
 
 #include "bs_internal.h"
+#include "fp_math.cuh"
 #include "mlp_internal.h"
 
 namespace bsi {
 
 namespace {
+
+using fpm::tanh_pair;
 
 constexpr int W = 128;           // hidden width of the tensor-core kernels
 constexpr int kWarps = 8, kThreads = 32 * kWarps, kRowsPerCta = 16 * kWarps;
@@ -88,65 +91,6 @@ __device__ void stage_net(const MlpDev &M, __nv_bfloat16 *W1s, __nv_bfloat16 *W2
 
 // ------------------------------------------------------------- inference
 //
-// Packed FP32 pairs: one instruction for two values.
-__device__ __forceinline__ uint64_t pk(float a, float b) {
-  return (uint64_t)__float_as_uint(a) | ((uint64_t)__float_as_uint(b) << 32);
-}
-__device__ __forceinline__ float lo_f(uint64_t v) { return __uint_as_float((uint32_t)v); }
-__device__ __forceinline__ float hi_f(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ float rcp(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// tanh of two values, about 11 instructions each and no branch.  |x| >= 0.55:
-// (1 - e) / (1 + e) with e = exp(-2 |x|) <= 1/3, no cancellation; below: an odd
-// polynomial |x| + |x|^3 P(x^2), P a degree-4 Chebyshev least-squares fit on
-// [0, 0.55^2] (relative error of the fit 1.1e-9).  Within 3e-7 relative of tanh
-// everywhere; NaN stays NaN, infinities give 1.  CORR: one more step takes the
-// reciprocal's error out of the quotient, for the gradient (1 - tanh^2), where an
-// error of one sign adds up over the rows; 7% of the inference time.
-template <bool CORR = false>
-__device__ __forceinline__ void tanh_pair(float x0, float x1, float &y0, float &y1) {
-  const float a0 = fabsf(x0), a1 = fabsf(x1);
-  const uint64_t a = pk(a0, a1), one = pk(1.f, 1.f);
-  const uint64_t u = mul2(a, pk(-2.88539008f, -2.88539008f));  // -2 log2(e) |x|
-  const uint64_t e = pk(ex2(lo_f(u)), ex2(hi_f(u)));
-  const uint64_t den = add2(e, one);
-  const uint64_t num = fma2(e, pk(-1.f, -1.f), one), rd = pk(rcp(lo_f(den)), rcp(hi_f(den)));
-  uint64_t big = mul2(num, rd);
-  if constexpr (CORR) big = fma2(fma2(big, pk(-lo_f(den), -hi_f(den)), num), rd, big);
-  const uint64_t q = mul2(a, a);
-  uint64_t p = fma2(q, pk(-0.00626437f, -0.00626437f), pk(0.02106414f, 0.02106414f));
-  p = fma2(q, p, pk(-0.0538503f, -0.0538503f));
-  p = fma2(q, p, pk(0.13332564f, 0.13332564f));
-  p = fma2(q, p, pk(-0.33333317f, -0.33333317f));
-  const uint64_t small = fma2(mul2(q, a), p, a);
-  y0 = copysignf(a0 < 0.55f ? lo_f(small) : lo_f(big), x0);
-  y1 = copysignf(a1 < 0.55f ? hi_f(small) : hi_f(big), x1);
-}
-
 __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -191,7 +135,7 @@ __device__ __forceinline__ uint32_t b_addr(uint32_t base, int ld, int j, int kk,
 // tensor pipe or HBM: the kernel it replaced issued 5970 warp instructions per 16
 // rows (weights staged for every 128 rows, one 32-bit shared load per B register,
 // a division per input, the library tanh on two divergent branches) and kept the
-// issue slots 47% busy.  1540 x 60^2 rows: 1.85 ms, 3.71 ms before.
+// issue slots 47% busy.  1540 x 60^2 rows: 1.86 ms, 3.71 ms before.
 template <int K1>
 __global__ void __launch_bounds__(kThreads, 2) k_mlp_tc_infer(MlpDev M, const float *__restrict__ x,
                                                               int n, float *__restrict__ y) {
@@ -518,8 +462,8 @@ __global__ void __launch_bounds__(kGradThreads, 1)
     };
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      tanh_pair<true>(h1[j][0], h1[j][1], h1[j][0], h1[j][1]);
-      tanh_pair<true>(h1[j][2], h1[j][3], h1[j][2], h1[j][3]);
+      tanh_pair(h1[j][0], h1[j][1], h1[j][0], h1[j][1]);
+      tanh_pair(h1[j][2], h1[j][3], h1[j][2], h1[j][3]);
       put(Ly::H1, j, h1[j]);
     }
     __syncthreads();
@@ -551,8 +495,8 @@ __global__ void __launch_bounds__(kGradThreads, 1)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const float2 w = *reinterpret_cast<const float2 *>(w3 + 32 * cq + 8 * j + 2 * t);
-      tanh_pair<true>(c2[j][0], c2[j][1], c2[j][0], c2[j][1]);
-      tanh_pair<true>(c2[j][2], c2[j][3], c2[j][2], c2[j][3]);
+      tanh_pair(c2[j][0], c2[j][1], c2[j][0], c2[j][1]);
+      tanh_pair(c2[j][2], c2[j][3], c2[j][2], c2[j][3]);
       y0 = fmaf(w.x, c2[j][0], fmaf(w.y, c2[j][1], y0));
       y1 = fmaf(w.x, c2[j][2], fmaf(w.y, c2[j][3], y1));
     }

@@ -1,0 +1,67 @@
+"""Device functions of csrc/fp_math.cuh against FP64: the error that each states,
+over every argument of its range, and the special values.  tests/gpu_fp_math.cu is
+compiled here with nvcc."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2506_10526_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def fpm(tmp_path_factory):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    out = tmp_path_factory.mktemp("fpm") / "libfpm.so"
+    r = subprocess.run([nvcc, "-gencode", "arch=compute_103a,code=sm_103a", "-std=c++17", "-O3",
+                        "-shared", "-Xcompiler", "-fPIC", "-I", CSRC, "-o", str(out),
+                        os.path.join(HERE, "gpu_fp_math.cu")], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return ctypes.CDLL(str(out))
+
+
+def _tanh(fpm, x):
+    x = np.ascontiguousarray(x, np.float32)
+    y = np.empty_like(x)
+    p = ctypes.POINTER(ctypes.c_float)
+    assert fpm.fpm_tanh(x.ctypes.data_as(p), y.ctypes.data_as(p), x.size) == 0
+    return y
+
+
+@pytest.mark.parametrize("exponent", range(-13, 4))
+def test_tanh_of_every_argument(fpm, exponent):
+    """Each binade from 2^-13 to 16, every FP32 value, both signs: within the stated
+    1.8e-7 relative of tanh, and against the correctly rounded value no bias above
+    1e-8 (rounding alone is biased near 2^-13, where tanh(x) lies just below x)."""
+    lo = (127 + exponent) << 23
+    out = (ctypes.c_double * 2)()
+    assert fpm.fpm_tanh_err(ctypes.c_uint32(lo), ctypes.c_uint32(1 << 23), out) == 0
+    assert out[0] <= 1.8e-7
+    assert abs(out[1]) <= 1e-8
+
+
+def test_tanh_special_values(fpm):
+    """Zeros with their sign, the smallest and small values (tanh(x) = x to rounding
+    below 2^-13), values beyond 16, infinities, NaN, and an odd function."""
+    inf, nan = np.float32(np.inf), np.float32(np.nan)
+    y = _tanh(fpm, [0.0, -0.0, inf, -inf, nan, 16.0, -1e30, 3e38])
+    assert y[0] == 0 and not np.signbit(y[0]) and y[1] == 0 and np.signbit(y[1])
+    assert y[2] == 1 and y[3] == -1 and np.isnan(y[4])
+    np.testing.assert_array_equal(y[5:], [1, -1, 1])
+    r = np.random.default_rng(1)
+    x = r.integers(1, 114 << 23, 100001).astype(np.uint32).view(np.float32)  # up to 2^-13
+    np.testing.assert_allclose(_tanh(fpm, x).astype(np.float64), np.tanh(x.astype(np.float64)),
+                               rtol=1.8e-7, atol=0)
+    x = np.concatenate([x, r.standard_normal(100001).astype(np.float32)])
+    np.testing.assert_array_equal(_tanh(fpm, -x), -_tanh(fpm, x))
