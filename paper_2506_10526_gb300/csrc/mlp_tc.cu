@@ -37,6 +37,8 @@ namespace bsi {
 
 namespace {
 
+using fpm::DivPair;
+using fpm::normalise_pair;
 using fpm::tanh_pair;
 
 constexpr int W = 128;           // hidden width of the tensor-core kernels
@@ -87,6 +89,19 @@ __device__ void stage_net(const MlpDev &M, __nv_bfloat16 *W1s, __nv_bfloat16 *W2
   for (int q = threadIdx.x; q < W; q += blockDim.x) b2[q] = p[q];
   p += W;
   for (int q = threadIdx.x; q < W; q += blockDim.x) w3[q] = __bfloat162float(__float2bfloat16_rn(p[q]));
+}
+
+// The normalisation of columns 2q and 2q + 1 in table entry q; columns beyond d pass zeros.
+template <int K1>
+__device__ void stage_norm(const MlpDev &M, DivPair *tab) {
+  for (int q = threadIdx.x; q < K1 / 2; q += blockDim.x) {
+    const int k = 2 * q, d = M.d;
+    DivPair t;
+    fpm::div_column(k < d ? M.norm[k] : 0.f, k < d ? M.norm[d + k] : 1.f, t.nmu.x, t.c.x, t.r.x, t.ns.x);
+    fpm::div_column(k + 1 < d ? M.norm[k + 1] : 0.f, k + 1 < d ? M.norm[d + k + 1] : 1.f, t.nmu.y, t.c.y,
+                    t.r.y, t.ns.y);
+    tab[q] = t;
+  }
 }
 
 // ------------------------------------------------------------- inference
@@ -144,7 +159,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp_tc_infer(MlpDev M, const fl
   __nv_bfloat16 *W1s = reinterpret_cast<__nv_bfloat16 *>(smem_raw);
   __nv_bfloat16 *W2s = W1s + W * LD1;
   float *b1 = reinterpret_cast<float *>(W2s + W * LD2), *b2 = b1 + W, *w3 = b2 + W;
-  float *mu = w3 + W, *inv = mu + K1, *xs = inv + K1;  // xs [128][d], 16-byte aligned
+  DivPair *norm = reinterpret_cast<DivPair *>(w3 + W);  // [K1 / 2]
+  float *xs = reinterpret_cast<float *>(norm + K1 / 2);  // [128][d], 16-byte aligned
   const int d = M.d, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
   const bool wide = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
@@ -165,10 +181,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp_tc_infer(MlpDev M, const fl
   };
   if (blockIdx.x < ntile) load(blockIdx.x);
   stage_net<K1>(M, W1s, W2s, b1, b2, w3);
-  for (int k = threadIdx.x; k < K1; k += kThreads) {
-    mu[k] = k < d ? M.norm[k] : 0.f;
-    inv[k] = k < d ? 1.f / M.norm[d + k] : 0.f;
-  }
+  stage_norm<K1>(M, norm);
   const float b3 = M.p[(long long)W * d + W + W * W + W + W];
   const float my = M.norm[2 * d], sy = M.norm[2 * d + 1];
   const uint32_t a1 = (uint32_t)__cvta_generic_to_shared(W1s), a2 = (uint32_t)__cvta_generic_to_shared(W2s);
@@ -184,10 +197,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp_tc_infer(MlpDev M, const fl
       for (int q = 0; q < 4; ++q) {  // a0: (g, 2t), a1: (g+8, 2t), a2: (g, 2t+8), a3: (g+8, 2t+8)
         const int col = 16 * kk + 2 * t + ((q >> 1) << 3);
         const float *xr = (q & 1) ? x1 : x0;
-        const float2 m2 = *reinterpret_cast<const float2 *>(mu + col);
-        const float2 i2 = *reinterpret_cast<const float2 *>(inv + col);
-        const float u0 = col < d ? (xr[col] - m2.x) * i2.x : 0.f;
-        const float u1 = col + 1 < d ? (xr[col + 1] - m2.y) * i2.y : 0.f;
+        float u0, u1;
+        normalise_pair(col < d ? xr[col] : 0.f, col + 1 < d ? xr[col + 1] : 0.f, norm[col / 2], u0, u1);
         split2(u0, u1, ah[kk][q], al[kk][q]);
       }
     }
@@ -326,8 +337,8 @@ struct GradLay {
   static constexpr int H1 = X + 2 * kGradRows * LD1 * 2;  // hi, lo [64][LD2]
   static constexpr int Z2 = H1 + 2 * kGradRows * LD2 * 2, Z1 = Z2 + 2 * kGradRows * LD2 * 2;
   static constexpr int vec = Z1 + 2 * kGradRows * LD2 * 2;
-  // gb1, gb2, gw3 [4][W], mu, inv [K1], yn parts [4][64], tn, ok [64], row [64], gb3
-  static constexpr int bytes = vec + (12 * W + 2 * K1 + 4 * kGradRows + 3 * kGradRows + 4) * 4;
+  // gb1, gb2, gw3 [4][W], norm [K1 / 2], yn parts [4][64], tn, ok [64], row [64], gb3
+  static constexpr int bytes = vec + (12 * W + 4 * K1 + 4 * kGradRows + 3 * kGradRows + 4) * 4;
 };
 
 // Loss and gradient of nrows rows (drawn as k_mlp_sample draws them when seeded:
@@ -357,8 +368,9 @@ __global__ void __launch_bounds__(kGradThreads, 1)
   static_assert(part_stride(K1) * 4 <= Ly::vec - Ly::X, "the partial gradient over the tile's buffers");
   extern __shared__ __align__(16) unsigned char sm[];
   const float *b1 = reinterpret_cast<const float *>(sm + Ly::net), *b2 = b1 + W, *w3 = b2 + W;
-  float *gb1 = reinterpret_cast<float *>(sm + Ly::vec), *gb2 = gb1 + 4 * W, *gw3 = gb2 + 4 * W, *mu = gw3 + 4 * W, *inv = mu + K1;
-  float *ypart = inv + K1, *tn = ypart + 4 * kGradRows, *okr = tn + kGradRows;
+  float *gb1 = reinterpret_cast<float *>(sm + Ly::vec), *gb2 = gb1 + 4 * W, *gw3 = gb2 + 4 * W;
+  DivPair *norm = reinterpret_cast<DivPair *>(gw3 + 4 * W);
+  float *ypart = reinterpret_cast<float *>(norm + K1 / 2), *tn = ypart + 4 * kGradRows, *okr = tn + kGradRows;
   int *rowid = reinterpret_cast<int *>(okr + kGradRows);
   float *gb3 = reinterpret_cast<float *>(rowid + kGradRows);
   const int d = M.d, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -370,10 +382,7 @@ __global__ void __launch_bounds__(kGradThreads, 1)
   pdl_launch();
   for (int q = tid; q < 12 * W; q += kGradThreads) gb1[q] = 0.f;
   if (tid == 0) *gb3 = 0.f;
-  for (int k = tid; k < K1; k += kGradThreads) {
-    mu[k] = k < d ? M.norm[k] : 0.f;
-    inv[k] = k < d ? 1.f / M.norm[d + k] : 0.f;
-  }
+  stage_norm<K1>(M, norm);
   float b3 = 0.f;
   const float my = M.norm[2 * d], sy = M.norm[2 * d + 1];
   float l2 = 0.f, sdy = 0.f;  // sums of squared residuals and of dyn
@@ -408,8 +417,7 @@ __global__ void __launch_bounds__(kGradThreads, 1)
       float v0 = 0.f, v1 = 0.f;
       if (row >= 0) {
         const float *xr = x + (long long)row * d;
-        if (c < d) v0 = (xr[c] - mu[c]) * inv[c];
-        if (c + 1 < d) v1 = (xr[c + 1] - mu[c + 1]) * inv[c + 1];
+        normalise_pair(c < d ? xr[c] : 0.f, c + 1 < d ? xr[c + 1] : 0.f, norm[c / 2], v0, v1);
       }
       uint32_t hi, lo;
       split2(v0, v1, hi, lo);
@@ -738,7 +746,7 @@ template <int K1>
 cudaError_t infer_k(const MlpDev &M, const float *x, int n, float *y, cudaStream_t s) {
   cudaError_t e = smem_optin_once<k_mlp_tc_infer<K1>>();
   if (e != cudaSuccess) return e;
-  const size_t sm = (size_t)W * (K1 + 8) * 2 + (size_t)W * LD2 * 2 + (3 * W + 2 * K1) * sizeof(float) +
+  const size_t sm = (size_t)W * (K1 + 8) * 2 + (size_t)W * LD2 * 2 + (3 * W + 4 * K1) * sizeof(float) +
                     (size_t)kRowsPerCta * M.d * sizeof(float);
   const int tiles = (n + kRowsPerCta - 1) / kRowsPerCta;
   k_mlp_tc_infer<K1><<<std::min(tiles, 2 * 152), kThreads, sm, s>>>(M, x, n, y);

@@ -34,9 +34,33 @@ __global__ void k_tanh_err(uint32_t lo, uint32_t n, unsigned long long *mx, doub
   atomicAdd(sum, s);
 }
 
+// u = (x - mu) / sd by pairs of columns, n rows of two
+__global__ void k_norm(const float *x, const float *mu, const float *sd, float *u, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  bsi::fpm::DivPair t;
+  bsi::fpm::div_column(mu[2 * i], sd[2 * i], t.nmu.x, t.c.x, t.r.x, t.ns.x);
+  bsi::fpm::div_column(mu[2 * i + 1], sd[2 * i + 1], t.nmu.y, t.c.y, t.r.y, t.ns.y);
+  bsi::fpm::normalise_pair(x[2 * i], x[2 * i + 1], t, u[2 * i], u[2 * i + 1]);
+}
+
 }  // namespace
 
 extern "C" {
+
+// in: x, mu, sd, 2 n values each; out: 2 n; host pointers
+int fpm_normalise(const float *in, float *out, int n) {
+  float *d = nullptr;
+  if (n < 1 || cudaMalloc(&d, 8 * (size_t)n * sizeof(float)) != cudaSuccess) return 1;
+  cudaError_t e = cudaMemcpy(d, in, 6 * (size_t)n * sizeof(float), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    k_norm<<<(n + 255) / 256, 256>>>(d, d + 2 * n, d + 4 * n, d + 6 * n, n);
+    e = cudaMemcpy(out, d + 6 * n, 2 * (size_t)n * sizeof(float), cudaMemcpyDeviceToHost);
+  }
+  cudaFree(d);
+  return e == cudaSuccess ? 0 : 1;
+}
+
 
 // y[n] = tanh(x[n]), host pointers
 int fpm_tanh(const float *x, float *y, int n) {

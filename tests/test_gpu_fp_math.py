@@ -65,3 +65,24 @@ def test_tanh_special_values(fpm):
                                rtol=1.8e-7, atol=0)
     x = np.concatenate([x, r.standard_normal(100001).astype(np.float32)])
     np.testing.assert_array_equal(_tanh(fpm, -x), -_tanh(fpm, x))
+
+
+@pytest.mark.parametrize("spread", [1.0, 60.0, 126.0, 149.0])
+def test_normalised_inputs_round_as_quotients(fpm, spread):
+    """(x - mu) / sd for ordinary deviations and for deviations up to 2^121 and down
+    to the smallest: never more than one unit in the last place from the division's
+    result, and equal to it in all but one in a thousand (the residual step rounds
+    as a division but where the remainder lies within the rounding of 1 / sd)."""
+    n = 1 << 19
+    r = np.random.default_rng(int(spread))
+    sd = (r.uniform(0.5, 2, 2 * n) * 2.0 ** r.uniform(-spread, min(spread, 120), 2 * n)).astype(np.float32)
+    sd[sd == 0] = np.float32(2.0 ** -149)
+    mu = (sd * r.standard_normal(2 * n)).astype(np.float32)
+    x = (mu + sd * r.standard_normal(2 * n)).astype(np.float32)
+    a = np.ascontiguousarray(np.concatenate([x, mu, sd]), np.float32)
+    got = np.empty(2 * n, np.float32)
+    p = ctypes.POINTER(ctypes.c_float)
+    assert fpm.fpm_normalise(a.ctypes.data_as(p), got.ctypes.data_as(p), n) == 0
+    want = (x - mu) / sd
+    assert np.all(np.abs(got.astype(np.float64) - want) <= np.spacing(np.abs(want)))
+    assert np.mean(got != want) <= 1e-3

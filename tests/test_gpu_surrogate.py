@@ -331,3 +331,30 @@ def test_column_statistics_of_the_largest_row_counts():
     f = 4000.0 / n
     mean, sd = 1.0 + 999.0 * f, 999.0 * np.sqrt(f * (1.0 - f))
     np.testing.assert_allclose(got, [mean, sd, mean, sd], rtol=2e-7)
+
+
+def test_inputs_are_divided_by_their_deviation():
+    """A deviation whose reciprocal overflows FP32 (2^-130): inputs that are that many
+    times small multiples of 2^-10 normalise exactly, so output and gradient equal,
+    bit for bit but for the order of sums, those of the multiples themselves."""
+    torch = _torch()
+    import paper_2506_10526_gb300 as bs
+    d, n, s = 20, 300, 2.0 ** -130
+    r = np.random.default_rng(3)
+    z = r.integers(-2048, 2049, (n, d)).astype(np.float32) / 1024
+    t = torch.from_numpy(r.standard_normal(n).astype(np.float32)).cuda()
+    res = []
+    for scale in (1.0, s):
+        net = bs.Surrogate(d, 128, seed=3)
+        p = net.params()
+        p[net.n_weights:net.n_weights + d] = 0.0
+        p[net.n_weights + d:net.n_weights + 2 * d] = scale
+        p[net.n_weights + 2 * d:] = [0.0, 1.0]
+        net.set_params(p)
+        x = torch.from_numpy((z.astype(np.float64) * scale).astype(np.float32)).cuda()
+        res.append((net.forward(x).cpu().numpy(), net.grad(x, t)))
+        net.close()
+    np.testing.assert_array_equal(res[0][0], res[1][0])
+    assert abs(res[0][1][0] - res[1][1][0]) <= 1e-6 * res[0][1][0]
+    np.testing.assert_allclose(res[0][1][1], res[1][1][1], rtol=0,
+                               atol=1e-6 * np.abs(res[0][1][1]).max())
