@@ -33,13 +33,30 @@ struct ColCfg {
   static constexpr int UB = N >= 256 ? 8 : 16;
 };
 
-constexpr int kRowThreads = 256;
-// row pairs per row-pass CTA for each side: at most one pass-2 transform (RPB N1) per
-// thread, which holds its outputs in registers while the exchange tile takes the rows
-template <int N>
+// The row pass, by image side and whether split BF16 rows are written beside the FP32
+// ones (HL).  Its stores bound it.  Straight from the last transform a warp's values
+// are runs of N1 floats and of N1 BF16s; put down in the exchange tile first (X), the
+// CTA's rows leave as whole 16-byte stores, for two barriers and a second trip through
+// shared memory.  Runs of 16 BF16s or 8 floats are whole sectors already.  Direct
+// against exchanged, us (FP32: 8 rings, 256 channels of 16 .. 128, 32 of 192 .. 768
+// pixels; BF16: 256 and 128 channels):
+//   side      16   24   32   48   64   96  128 |  192  256  384  512  768
+//   FP32     4.1  6.1  8.2 11.8 15.1 32.7 61.5 | 17.2   23   75  106  270
+//            3.5  5.3  6.6 12.3 15.8 37.4 57.4 | 18.5   29   85  125  327
+//   + BF16   5.5  9.2   15   23   28   64  106 |  135  125  358  548 1606
+//            3.8  5.8  7.3   14   19   46   72 |   83  144  349  566 1439
+// (32 channels: exchanged 48 and 64 take 4.9 and 5.0 us in FP32, direct 5.8 and 5.6.)
+// So split BF16 rows go through the tile where a run of N1 is no whole sector, FP32
+// rows alone up to 64 pixels and at 128.
+template <int N, bool HL>
 struct RowCfg {
-  static constexpr int RPB = N <= 32 ? 64 : N == 48 ? 42 : N <= 128 ? 32 : N == 192 ? 21
-                           : N == 768 ? 10 : 16;
+  static constexpr bool X = HL ? Split<N>::N1 % 16 != 0 : N <= 64 || N == 128;
+  static constexpr int THREADS = X ? 256 : kRegThreads;
+  // row pairs per CTA.  X: at most one pass-2 transform (RPB N1) per thread, which
+  // holds its outputs in registers while the exchange tile takes the rows; direct:
+  // about one or two, in whole warps
+  static constexpr int RPB = X ? (N <= 32 ? 64 : N == 48 ? 42 : N <= 128 ? 32 : N == 192 ? 21 : 10)
+                               : (N <= 128 ? 32 : N == 192 ? 16 : 8);
 };
 
 __device__ __forceinline__ uint16_t bf16_bits_r(float x) {
@@ -135,13 +152,29 @@ __global__ void __launch_bounds__(kRegThreads) k_colpass_reg(
   }
 }
 
-template <int N>
-__global__ void __launch_bounds__(kRowThreads) k_rowpass_reg(
+// The largest |F| of the values that the warp's lanes hold (amax: float bits; key: the
+// lane's (realisation, slot), -1 in a lane without values), for the split FP16 scales.
+// Lanes without values lie behind all others and follow the first lane's key: without
+// that the last warp of every block of 48, 192 or 768 pixels sent one atomic per lane (192
+// pixels, 64 channels: 67 us, 31 with it).
+__device__ __forceinline__ void row_max(unsigned *fmax, int key, unsigned amax) {
+  const int k0 = __shfl_sync(0xffffffffu, key, 0);
+  if (__all_sync(0xffffffffu, key == k0 || key < 0)) {  // one (realisation, slot) in the warp
+    amax = __reduce_max_sync(0xffffffffu, key < 0 ? 0u : amax);
+    if ((threadIdx.x & 31) == 0 && k0 >= 0 && amax) atomicMax(fmax + k0, amax);
+  } else if (key >= 0 && amax) {
+    atomicMax(fmax + key, amax);
+  }
+}
+
+// fmax only without the split BF16 rows (HL).
+template <int N, bool HL>
+__global__ void __launch_bounds__(RowCfg<N, HL>::THREADS) k_rowpass_reg(
     GridGeom g, long long npairs, const float2 *__restrict__ G, const uint8_t *__restrict__ valid,
     const int *__restrict__ uext, const float2 *__restrict__ twM, float *__restrict__ F,
     uint16_t *__restrict__ Fhi, uint16_t *__restrict__ Flo, unsigned *__restrict__ fmax) {
   constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2, LDY = Split<N>::LDY;
-  constexpr int RPB = RowCfg<N>::RPB, HALF = N / 2;
+  constexpr int RPB = RowCfg<N, HL>::RPB, HALF = N / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2 *tw2 = reinterpret_cast<float2 *>(smem_raw);  // [N1][N2]
   float2 *Y = tw2 + N;                                   // [RPB][N1][LDY]
@@ -210,74 +243,97 @@ __global__ void __launch_bounds__(kRowThreads) k_rowpass_reg(
     }
   }
   __syncthreads();
-  // pass 2: (pair, k1) items, k1 fastest; outputs X[k1 + N1 k2], put down in the
-  // exchange tile (each thread has read its part) as the CTA's 2 RPB rows of F, which
-  // are contiguous.  Stores bound the pass: straight from here a warp's values are
-  // runs of N1 floats (32 bytes for N = 96) and of N1 BF16s (16 bytes), a partial
-  // sector each; from the tile they are whole 16-byte stores.  Per launch, 256 channels
-  // of 192 / 128 / 96 pixels: 544 -> 335, 196 -> 123, 118 -> 81 us; 128 Monte Carlo
-  // realisations of 96 / 64 / 48: 920 -> 597, 393 -> 258, 312 -> 127 us; sides of 256
-  // and more, whose runs were whole sectors already, within 6% either way.
-  constexpr int PAD = (N1 + 3) / 4 * 4, PO = 2 * N + PAD;  // floats of a row pair: lanes on their own banks
-  static_assert(RPB * N1 <= kRowThreads, "one item per thread");
-  static_assert(RPB * PO <= RPB * N1 * LDY * 2, "rows over the exchange tile");
-  float *out = reinterpret_cast<float *>(Y);
-  {
-    const int it = threadIdx.x;
-    const int r = it / N1, k1 = it - r * N1;
-    const bool mine = it < RPB * N1, live = mine && q0 + r < npairs;
-    float2 v[N2];
-    if (mine) {
+  if constexpr (!RowCfg<N, HL>::X) {
+    // pass 2: (pair, k1) items, k1 fastest; outputs X[k1 + N1 k2] -> columns
+    static_assert(RPB * N1 % 32 == 0, "whole warps in every step (row_max)");
+    for (int it = threadIdx.x; it < RPB * N1; it += blockDim.x) {
+      const int r = it / N1, k1 = it - r * N1;
+      const long long q = q0 + r;
+      const bool live = q < npairs;
+      float2 v[N2];
       const float2 *Yr = Y + r * (N1 * LDY) + k1 * LDY;
 #pragma unroll
       for (int n2 = 0; n2 < N2; ++n2) v[n2] = Yr[n2];
-    }
-    __syncthreads();
-    unsigned amax = 0;
-    if (mine) {
       freg::dft<N2, 1>(v);
+      unsigned amax = 0;
+      if (live) {
+        // F rows 2p, 2p + 1 of field fq = q / HALF: offset (2 q) N
+        const long long o0 = 2 * q * N, o1 = o0 + N;
 #pragma unroll
-      for (int k2 = 0; k2 < N2; ++k2) {
-        float *o = out + r * PO + k1 + N1 * k2;
-        o[0] = v[k2].x;
-        o[N] = v[k2].y;
-        amax = max(amax, __float_as_uint(fmaxf(fabsf(v[k2].x), fabsf(v[k2].y))));
+        for (int k2 = 0; k2 < N2; ++k2) {
+          const int x = k1 + N1 * k2;
+          const float a = v[k2].x, c = v[k2].y;
+          if (!BS_CHK(o1 + x, 2 * npairs * N, 4)) continue;
+          F[o0 + x] = a;
+          F[o1 + x] = c;
+          amax = max(amax, __float_as_uint(fmaxf(fabsf(a), fabsf(c))));
+          if constexpr (HL) {
+            const uint16_t ha = bf16_bits_r(a), hc = bf16_bits_r(c);
+            Fhi[o0 + x] = ha;
+            Fhi[o1 + x] = hc;
+            Flo[o0 + x] = bf16_bits_r(a - bf16_val_r(ha));
+            Flo[o1 + x] = bf16_bits_r(c - bf16_val_r(hc));
+          }
+        }
       }
+      if (!HL && fmax) row_max(fmax, live ? key_s[r] : -1, amax);
     }
-    if (fmax) {
-      const int key = live ? key_s[r] : -1;
-      const int k0 = __shfl_sync(0xffffffffu, key, 0);
-      if (__all_sync(0xffffffffu, key == k0)) {  // one (realisation, slot) in the warp
-        amax = __reduce_max_sync(0xffffffffu, amax);
-        if ((threadIdx.x & 31) == 0 && k0 >= 0 && amax) atomicMax(fmax + k0, amax);
-      } else if (key >= 0 && amax) {
-        atomicMax(fmax + key, amax);
-      }
-    }
-    __syncthreads();
-  }
-  for (int e = threadIdx.x; e < RPB * (N / 4); e += blockDim.x) {  // 8 pixels each
-    const int r = e / (N / 4), x = 8 * (e - r * (N / 4));
-    if (q0 + r >= npairs) break;
-    const long long o = 2 * (q0 + r) * N + x;
-    if (!BS_CHK(o + 7, 2 * npairs * N, 4)) continue;
-    const float4 u0 = *reinterpret_cast<const float4 *>(out + r * PO + x);
-    const float4 u1 = *reinterpret_cast<const float4 *>(out + r * PO + x + 4);
-    *reinterpret_cast<float4 *>(F + o) = u0;
-    *reinterpret_cast<float4 *>(F + o + 4) = u1;
-    if (Fhi) {
-      const float u[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-      uint32_t hi[4], lo[4];
+  } else {
+    // pass 2: (pair, k1) items, k1 fastest; outputs X[k1 + N1 k2], put down in the
+    // exchange tile (each thread has read its part) as the CTA's 2 RPB rows of F, which
+    // are contiguous
+    constexpr int PAD = (N1 + 3) / 4 * 4, PO = 2 * N + PAD;  // floats of a row pair: lanes on their own banks
+    static_assert(RPB * N1 <= RowCfg<N, HL>::THREADS, "one item per thread");
+    static_assert(RPB * PO <= RPB * N1 * LDY * 2, "rows over the exchange tile");
+    float *out = reinterpret_cast<float *>(Y);
+    {
+      const int it = threadIdx.x;
+      const int r = it / N1, k1 = it - r * N1;
+      const bool mine = it < RPB * N1, live = mine && q0 + r < npairs;
+      float2 v[N2];
+      if (mine) {
+        const float2 *Yr = Y + r * (N1 * LDY) + k1 * LDY;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint16_t h0 = bf16_bits_r(u[2 * k]), h1 = bf16_bits_r(u[2 * k + 1]);
-        const uint16_t l0 = bf16_bits_r(u[2 * k] - bf16_val_r(h0)),
-                       l1 = bf16_bits_r(u[2 * k + 1] - bf16_val_r(h1));
-        hi[k] = (uint32_t)h0 | ((uint32_t)h1 << 16);
-        lo[k] = (uint32_t)l0 | ((uint32_t)l1 << 16);
+        for (int n2 = 0; n2 < N2; ++n2) v[n2] = Yr[n2];
       }
-      *reinterpret_cast<uint4 *>(Fhi + o) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-      *reinterpret_cast<uint4 *>(Flo + o) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+      __syncthreads();
+      unsigned amax = 0;
+      if (mine) {
+        freg::dft<N2, 1>(v);
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) {
+          float *o = out + r * PO + k1 + N1 * k2;
+          o[0] = v[k2].x;
+          o[N] = v[k2].y;
+          amax = max(amax, __float_as_uint(fmaxf(fabsf(v[k2].x), fabsf(v[k2].y))));
+        }
+      }
+      if (!HL && fmax) row_max(fmax, live ? key_s[r] : -1, amax);
+      __syncthreads();
+    }
+    for (int e = threadIdx.x; e < RPB * (N / 4); e += blockDim.x) {  // 8 pixels each
+      const int r = e / (N / 4), x = 8 * (e - r * (N / 4));
+      if (q0 + r >= npairs) break;
+      const long long o = 2 * (q0 + r) * N + x;
+      if (!BS_CHK(o + 7, 2 * npairs * N, 4)) continue;
+      const float4 u0 = *reinterpret_cast<const float4 *>(out + r * PO + x);
+      const float4 u1 = *reinterpret_cast<const float4 *>(out + r * PO + x + 4);
+      *reinterpret_cast<float4 *>(F + o) = u0;
+      *reinterpret_cast<float4 *>(F + o + 4) = u1;
+      if constexpr (HL) {
+        const float u[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint16_t h0 = bf16_bits_r(u[2 * k]), h1 = bf16_bits_r(u[2 * k + 1]);
+          const uint16_t l0 = bf16_bits_r(u[2 * k] - bf16_val_r(h0)),
+                         l1 = bf16_bits_r(u[2 * k + 1] - bf16_val_r(h1));
+          hi[k] = (uint32_t)h0 | ((uint32_t)h1 << 16);
+          lo[k] = (uint32_t)l0 | ((uint32_t)l1 << 16);
+        }
+        *reinterpret_cast<uint4 *>(Fhi + o) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        *reinterpret_cast<uint4 *>(Flo + o) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+      }
     }
   }
 }
@@ -302,20 +358,20 @@ cudaError_t colpass_n(const GridGeom &g, const float2 *vis, const float *ngrid,
   return cudaGetLastError();
 }
 
-template <int N>
+template <int N, bool HL>
 cudaError_t rowpass_n(const GridGeom &g, const float2 *G, const uint8_t *valid, const int *uext,
                       const float2 *twM, float *F, uint16_t *Fhi, uint16_t *Flo, unsigned *fmax,
                       cudaStream_t s) {
-  constexpr int RPB = RowCfg<N>::RPB;
-  const size_t smem = (size_t)(N + RPB * Split<N>::N1 * Split<N>::LDY) * sizeof(float2);
-  cudaError_t e = smem_optin_once<k_rowpass_reg<N>>();
+  using Cfg = RowCfg<N, HL>;
+  const size_t smem = (size_t)(N + Cfg::RPB * Split<N>::N1 * Split<N>::LDY) * sizeof(float2);
+  cudaError_t e = smem_optin_once<k_rowpass_reg<N, HL>>();
   if (e != cudaSuccess) return e;
   const long long npairs = (long long)g.batch * g.nslot * g.nc * (N / 2);
   if (npairs == 0) return cudaSuccess;
-  const long long nblk = (npairs + RPB - 1) / RPB;
+  const long long nblk = (npairs + Cfg::RPB - 1) / Cfg::RPB;
   if (nblk > 0x7fffffffLL) return cudaErrorInvalidValue;
-  k_rowpass_reg<N><<<(unsigned)nblk, kRowThreads, smem, s>>>(g, npairs, G, valid, uext, twM, F,
-                                                             Fhi, Flo, fmax);
+  k_rowpass_reg<N, HL><<<(unsigned)nblk, Cfg::THREADS, smem, s>>>(g, npairs, G, valid, uext, twM, F,
+                                                                  Fhi, Flo, fmax);
   return cudaGetLastError();
 }
 
@@ -352,7 +408,9 @@ cudaError_t launch_rowpass_reg(const GridGeom &g, const float2 *G, const uint8_t
                                uint16_t *Flo, unsigned *fmax, cudaStream_t s) {
   switch (g.M) {
 #define BS_ROW_CASE(n) \
-  case n: return rowpass_n<n>(g, G, valid, uext, twM, F, Fhi, Flo, fmax, s);
+  case n:                                                                       \
+    return Fhi ? rowpass_n<n, true>(g, G, valid, uext, twM, F, Fhi, Flo, fmax, s) \
+               : rowpass_n<n, false>(g, G, valid, uext, twM, F, Fhi, Flo, fmax, s);
     BS_REG_SIDES(BS_ROW_CASE)
 #undef BS_ROW_CASE
     default: return cudaErrorInvalidValue;

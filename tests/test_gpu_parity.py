@@ -496,3 +496,35 @@ def test_every_register_transform_side(cmax, side):
             ok = ~np.isnan(want)
             assert np.array_equal(np.isnan(got[k]), ~ok)
             assert np.all(np.abs(got[k][ok] - want[ok]) <= TOL[precision] * size[ok])
+
+
+@pytest.mark.parametrize("cmax,side", [(5, 16), (15, 48), (31, 96), (63, 192), (85, 256), (255, 768)])
+def test_split_fp16_of_register_transform_sides(cmax, side):
+    """Split FP16, whose row pass writes FP32 rows alone and takes the largest value of
+    each (realisation, ring): sides that go through the exchange tile and sides that
+    do not, whole and part-filled last warps (48, 192, 768), blocks of rows over two
+    rings.  Realisations and rings of very different size, so that a maximum of
+    another ring or of an idle lane shows as a lost or an overflowing scale."""
+    torch = _torch()
+    import paper_2506_10526_gb300 as bs
+    nt, nc, edges = 2 * cmax + 2, 3, [1.0, 2.3, cmax - 0.6, cmax + 0.2]
+    vis = np.stack([synth.sky_visibilities(nt, nc, seed=side + k) for k in range(2)])
+    vis[1] *= 1e-3
+    c = np.arange(nt) - nt // 2
+    vis[:, :, np.hypot(*np.meshgrid(c, c)) > 3] *= 1e3
+    trips = [(0, 0, 0), (0, 2, 2), (2, 2, 2)]
+    index = [oracle.ring_triples(3).index(t) for t in trips]
+    plan = bs.Plan(nt, nc, edges, precision=2, batch=2)
+    assert plan.M == side
+    plan.grid_load(torch.from_numpy(vis.astype(np.complex64)).cuda())
+    full = torch.empty((2, plan.ntrip, nc, nc, nc), dtype=torch.float64, device="cuda")
+    plan.mabs(out_full=full)
+    torch.cuda.synchronize()
+    got = full.cpu().numpy()[:, index]
+    plan.close()
+    for k, v in enumerate(vis):
+        want = oracle.mabs_full(v, edges, triples=trips)["B"].real
+        size = oracle.mabs_full(np.abs(v), edges, triples=trips)["B"].real
+        ok = ~np.isnan(want)
+        assert np.array_equal(np.isnan(got[k]), ~ok)
+        assert np.all(np.abs(got[k][ok] - want[ok]) <= TOL[2] * size[ok])
