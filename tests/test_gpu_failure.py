@@ -125,3 +125,57 @@ def test_injected_allocation_failures_are_reported_cleanly():
         assert tag in out, out
     line = [l for l in out.splitlines() if l.startswith("AFTER")][0].split()
     assert line[1] == "True" and float(line[2]) < 1e-5, out
+
+
+CHILD_PAIR = textwrap.dedent("""
+    import os, sys, numpy as np, torch
+    sys.path.insert(0, ROOT)
+    import paper_2506_10526_gb300 as bs, synth
+    nc, precision, with_full = NC, PREC, FULL
+    vis = torch.from_numpy(synth.sky_visibilities(32, nc, seed=1)[None]).cuda()
+    edges = synth.edges_linear(3, 16)
+    out = torch.empty((1, 10, 2 * nc - 1, 2 * nc - 1), dtype=torch.float64, device="cuda")
+    full = torch.empty((1, 10, nc, nc, nc), dtype=torch.float64, device="cuda") if with_full else None
+    plan = bs.Plan(32, nc, edges, precision=precision)
+    plan.grid_load(vis)
+    for stall in "101":
+        os.environ["BS_INJECT_MMA_STALL"] = stall
+        plan.grid_load(vis)
+        plan.delta_reset()
+        plan.mabs(out_full=full)
+        try:
+            plan.mabs_delta(out)
+            torch.cuda.synchronize()
+            print("DONE", stall)
+        except bs.BsError as e:
+            print("STATUS", stall, e.status)
+        if stall == "0":
+            got = out.cpu().numpy()
+    ref = bs.Plan(32, nc, edges)
+    ref.grid_load(vis)
+    ref.mabs()
+    ref.mabs_delta(out)
+    torch.cuda.synchronize()
+    want = out.cpu().numpy()
+    ok = ~np.isnan(want)
+    rel = np.abs(got[ok] - want[ok]).max() / np.abs(want[ok]).max()
+    print("RECOVERED", bool(np.array_equal(np.isnan(got), ~ok)) and rel < 1e-3, rel)
+""").replace("ROOT", repr(ROOT))
+
+
+@pytest.mark.parametrize("nc,full", [(4, True), (128, False)])
+@pytest.mark.parametrize("precision", [1, 2])
+def test_bounded_waits_of_the_two_sm_contraction(nc, full, precision):
+    """The same for the contraction kernel of two SMs a tile, which the small case
+    above no longer reaches: a call that also writes the uncollapsed bins always takes
+    it, and so does a collapse whose column windows are full (its epilogue's warps
+    then take the chunks in step).  Time-out, a normal run, time-out again."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    src = CHILD_PAIR.replace("NC, PREC, FULL", f"{nc}, {precision}, {full}")
+    r = subprocess.run([sys.executable, "-c", src], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    lines = r.stdout.splitlines()
+    assert lines[:3] == ["STATUS 1 6", "DONE 0", "STATUS 1 6"], r.stdout  # 6: BS_ERR_TIMEOUT
+    assert "RECOVERED True" in r.stdout, r.stdout
