@@ -340,3 +340,45 @@ def test_statistics_of_every_batch_form(batch):
         want_v = ref[:, ok].var(axis=0, ddof=1)
         assert np.all(np.abs(mean[ok] - ref[:, ok].mean(axis=0)) <= tol)
         assert np.all(np.abs(var[ok] - want_v) <= 2 * np.sqrt(want_v) * tol + tol ** 2)
+
+
+@pytest.mark.parametrize("precision", [1, 2])
+@pytest.mark.parametrize("nc", [5, 8, 16])
+def test_both_contractions_give_the_same_sums(nc, precision):
+    """A group of at most 16 channels runs through the contraction for short column
+    lists; next to a group of more channels the whole ensemble runs through the
+    two-SM contraction, with the same tiles for the small group (K split by its own
+    tiles).  Where each entry is summed by one warp the FP32 sums are the same bits,
+    and what is left is the order of at most a few hundred FP64 sums: 1e-12 of the
+    largest value (an FP32 sum in another order differs by 1e-8)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2506_10526_gb300 as bs
+    small = dict(nt=24, nchan=nc, edges=list(synth.edges_linear(5, 12)), batch=3,
+                 precision=precision, multires=True)
+    large = dict(nt=16, nchan=20, edges=list(synth.edges_linear(2, 8)), batch=1,
+                 precision=precision)
+    flags = np.zeros(nc, np.uint8)
+    flags[nc // 2] = 1
+
+    def run(groups):
+        ens = bs.Ensemble(groups)
+        bufs = []
+        for g, spec in enumerate(groups):
+            v = np.stack([synth.sky_visibilities(spec["nt"], spec["nchan"], 50 + k)
+                          for k in range(spec["batch"])])
+            bufs.append(torch.from_numpy(v.astype(np.complex64)).cuda())
+            ens.set_input(g, bufs[g])
+        ens.set_flags(0, flags)
+        ens.run(use_graph=False)
+        out = ens.stats(0, 0)
+        ens.close()
+        return out
+
+    alone, beside = run([small]), run([small, large])
+    for a, b in zip(alone[:2], beside[:2]):
+        assert np.array_equal(np.isnan(a), np.isnan(b))
+        ok = ~np.isnan(a)
+        assert ok.any() and np.abs(a[ok]).max() > 0
+        assert np.abs(a[ok] - b[ok]).max() <= 1e-12 * np.abs(a[ok]).max()
