@@ -38,6 +38,7 @@
 #include <limits>
 #include <vector>
 
+#include "fp_math.cuh"
 #include "plan_internal.h"
 
 namespace bsi {
@@ -265,18 +266,6 @@ static void mono_split(MonoArgs &a, int npl, int nrows, int &gx) {
   gx = (ncw * nrc + kThreads / 32 - 1) / (kThreads / 32);
 }
 
-// 1 / sqrt(s) in FP64 for s in FP32's normal range: an FP32 seed (relative error
-// below 2^-19: the 20 leading mantissa bits of s, then rsqrtf) and one third-order
-// step, y (1 + e / 2 + 3 e^2 / 8) with e = 1 - s y^2, whose error 5 e^3 / 16 is below
-// 2^-55.  Five FP64 operations, against a square root and a division.
-__device__ __forceinline__ double rsqrt64(double s) {
-  const uint32_t h = (uint32_t)__double2hiint(s);
-  const uint32_t f = __float_as_uint(rsqrtf(__uint_as_float((h - (896u << 20)) << 3)));
-  const double y = __hiloint2double((int)((f >> 3) + (896u << 20)), (int)(f << 29));
-  const double e = __fma_rn(-__dmul_rn(s, y), y, 1.0);
-  return __fma_rn(__dmul_rn(y, e), __fma_rn(0.375, e, 0.5), y);
-}
-
 // m = 0 multipoles (Eq. bs_lm): per bin the sums of (2l+1) P_l(mu_1) B over the
 // paired samples, l = 0..LMAX, with mu_1 = k_par / k of the largest side (the
 // first of sides 1, 2, 3 on ties; sides as the oracle rounds them).  Bins come
@@ -378,7 +367,7 @@ __global__ void __launch_bounds__(kThreads) k_mono_multipole(const MonoArgs a,
           double sm = s1, zm = za;
           if (__double_as_longlong(s2) > __double_as_longlong(sm)) { sm = s2; zm = zb; }
           if (__double_as_longlong(s3) > __double_as_longlong(sm)) { sm = s3; zm = zc; }
-          x = __dmul_rn(zm, rsqrt64(sm));
+          x = __dmul_rn(zm, fpm::rsqrt64(sm));
           if (LMAX >= 2) x2 = __dmul_rn(x, x);
         }
         const double w2 = LMAX >= 2 ? __fma_rn(7.5, x2, -2.5) : 0.0;

@@ -44,9 +44,28 @@ __global__ void k_norm(const float *x, const float *mu, const float *sd, float *
   bsi::fpm::normalise_pair(x[2 * i], x[2 * i + 1], t, u[2 * i], u[2 * i + 1]);
 }
 
+__global__ void k_rsqrt(const double *s, double *y, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) y[i] = bsi::fpm::rsqrt64(s[i]);
+}
+
 }  // namespace
 
 extern "C" {
+
+// y[n] = 1 / sqrt(s[n]), host pointers
+int fpm_rsqrt(const double *s, double *y, int n) {
+  double *d = nullptr;
+  if (n < 1 || cudaMalloc(&d, 2 * (size_t)n * sizeof(double)) != cudaSuccess) return 1;
+  cudaError_t e = cudaMemcpy(d, s, (size_t)n * sizeof(double), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    k_rsqrt<<<(n + 255) / 256, 256>>>(d, d + n, n);
+    e = cudaMemcpy(y, d + n, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost);
+  }
+  cudaFree(d);
+  return e == cudaSuccess ? 0 : 1;
+}
+
 
 // in: x, mu, sd, 2 n values each; out: 2 n; host pointers
 int fpm_normalise(const float *in, float *out, int n) {

@@ -86,3 +86,20 @@ def test_normalised_inputs_round_as_quotients(fpm, spread):
     want = (x - mu) / sd
     assert np.all(np.abs(got.astype(np.float64) - want) <= np.spacing(np.abs(want)))
     assert np.mean(got != want) <= 1e-3
+
+
+def test_reciprocal_square_root(fpm):
+    """Squared lengths from the smallest to the largest that the binnings accept (k_perp
+    in [1e-8, 1e8], |k_par| up to 1e8: 1e-16 to 5e16), over FP32's normal range, at
+    powers of two and their neighbours: below 2^-52 relative, against extended
+    precision."""
+    r = np.random.default_rng(4)
+    two = 2.0 ** np.arange(-126, 128)
+    s = np.concatenate([10.0 ** r.uniform(-16, np.log10(5e16), 1 << 20), [1e-16, 5e16],
+                        two * r.uniform(1, 2, two.size), two, np.nextafter(two[1:], 0),
+                        np.nextafter(two, np.inf)])
+    y = np.empty_like(s)
+    p = ctypes.POINTER(ctypes.c_double)
+    assert fpm.fpm_rsqrt(s.ctypes.data_as(p), y.ctypes.data_as(p), s.size) == 0
+    want = 1 / np.sqrt(s.astype(np.longdouble))
+    assert np.abs(y / want - 1).max() < 2.0 ** -52
