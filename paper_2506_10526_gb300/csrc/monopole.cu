@@ -143,37 +143,45 @@ __global__ void __launch_bounds__(kThreads) k_mono_bins(const MonoArgs a, long l
 // for the whole warp, nearly every group of 32 samples was mixed where the bins
 // are narrow along b, and went sample by sample through FP64 shared-memory
 // atomics (compare-and-swap loops): 3.34 ms for 216 planes of 768^2 (12 x 5 x 5
-// bins) against 0.43 ms now, 2.9 TB/s of bins and values (the FP64 adds alone
+// bins) against 0.44 ms now, 2.8 TB/s of bins and values (the FP64 adds alone
 // take 0.24 ms).
 //
 // Adds x[0..NX) of the lanes in `who` (a ballot; each lane's own bin `cur`) to the
 // histogram rows hs[k * nbin + cur], and their counts.  Called by the whole
-// warp.  Lanes that close the same bin are summed by shuffles first: their
-// atomics would serialise on one address.
+// warp.  Lanes that close the same bin are summed by shuffles first where there are more
+// than eight of them (their atomics serialise on one address); the others add their
+// own, all at once: with narrow bins every lane closes another bin on every row.  Bin
+// after bin through the shuffles, 170 planes of 32^2 in 40 x 10 x 10 bins, four
+// realisations, took 387 us against 104 of the row walk; 79 now (calls, with their
+// launches; more than two lanes instead of eight: 90).
 template <int NX>
 __device__ __forceinline__ void flush_lanes(unsigned who, int cur, const double *x, unsigned cnt,
                                             int nx, int nbin, double *hs, unsigned *hc, int lane) {
-  while (who) {
-    const int bin = __shfl_sync(0xffffffffu, cur, __ffs(who) - 1);
-    const bool mine = ((who >> lane) & 1u) && cur == bin;
-    const unsigned grp = __ballot_sync(0xffffffffu, mine);
-    who &= ~grp;
-    if (__popc(grp) > 2) {
-      unsigned c = mine ? cnt : 0u;
-      for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-      if (lane == 0) atomicAdd(hc + bin, c);
+  const bool in = (who >> lane) & 1u;
+  unsigned peers = 0;
+  if (in) peers = __match_any_sync(who, cur);
+  const bool many = __popc(peers) > 8;
+  if (in && !many) {
+    atomicAdd(hc + cur, cnt);
 #pragma unroll
-      for (int k = 0; k < NX; ++k) {
-        if (k >= nx) break;
-        double v = mine ? x[k] : 0.0;
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) atomicAdd(hs + (size_t)k * nbin + bin, v);
-      }
-    } else if (mine) {
-      atomicAdd(hc + bin, cnt);
+    for (int k = 0; k < NX; ++k)
+      if (k < nx) atomicAdd(hs + (size_t)k * nbin + cur, x[k]);
+  }
+  unsigned rest = __ballot_sync(0xffffffffu, many);
+  while (rest) {
+    const unsigned grp = __shfl_sync(0xffffffffu, peers, __ffs(rest) - 1);
+    const int bin = __shfl_sync(0xffffffffu, cur, __ffs(rest) - 1);
+    const bool mine = (grp >> lane) & 1u;
+    rest &= ~grp;
+    unsigned c = mine ? cnt : 0u;
+    for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (lane == 0) atomicAdd(hc + bin, c);
 #pragma unroll
-      for (int k = 0; k < NX; ++k)
-        if (k < nx) atomicAdd(hs + (size_t)k * nbin + bin, x[k]);
+    for (int k = 0; k < NX; ++k) {
+      if (k >= nx) break;
+      double v = mine ? x[k] : 0.0;
+      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) atomicAdd(hs + (size_t)k * nbin + bin, v);
     }
   }
 }
@@ -256,14 +264,18 @@ __global__ void __launch_bounds__(kThreads) k_mono_sum(const MonoArgs a,
 
 // Rows and units of the column-walking kernels over nrows rows: as many row
 // ranges per plane as fill the chip about three times over with 32 warps per
-// SM, at least 32 rows each (a range's end flushes every lane).
+// SM, at least 32 rows each (a range's end flushes every lane), and where the columns
+// do not give every warp of a CTA a unit, ranges of down to two rows that do: one
+// range for planes of 32^2 left seven warps of eight idle (multipoles of 170 such planes,
+// 8 realisations, shifted axis: 809 us with the row walk, 1715 so, 310 now).
 static void mono_split(MonoArgs &a, int npl, int nrows, int &gx) {
-  const int ncw = (a.nc + 31) / 32;
+  const int ncw = (a.nc + 31) / 32, nw = kThreads / 32;
   const long long units = (long long)npl * ncw;
-  const int want = (int)std::min<long long>(std::max(1, nrows / 32), (3LL * 152 * 32 + units - 1) / units);
+  const int fill = std::max(1, std::min(nrows / 2, (nw + ncw - 1) / ncw));
+  const int want = std::max<int>(fill, (int)std::min<long long>(std::max(1, nrows / 32), (3LL * 152 * 32 + units - 1) / units));
   a.chunk = (nrows + want - 1) / want;
   const int nrc = (nrows + a.chunk - 1) / a.chunk;
-  gx = (ncw * nrc + kThreads / 32 - 1) / (kThreads / 32);
+  gx = (ncw * nrc + nw - 1) / nw;
 }
 
 // m = 0 multipoles (Eq. bs_lm): per bin the sums of (2l+1) P_l(mu_1) B over the
