@@ -68,11 +68,13 @@ constexpr double kU = 1.0 / 16777216.0;  // 2^-24
 constexpr int kNormThreads = 512;
 
 // The FP32 fields of every level: level q holds fields first[q] .. first[q + 1] - 1
-// of m2[q] pixels.
+// of m2[q] pixels.  NL: 1 for plans of one image side, whose calls are small (the
+// arguments of kMaxLevels levels add some 2 us to a launch), or kMaxLevels.
+template <int NL>
 struct NormLevels {
-  const float *F[kMaxLevels];
-  long long m2[kMaxLevels];
-  int first[kMaxLevels + 1];
+  const float *F[NL];
+  long long m2[NL];
+  int first[NL + 1];
 };
 
 // Per-field norms: out[3 f + 0..2] = max |F|, ||F||_2, ||F||_3.  One CTA per
@@ -80,8 +82,9 @@ struct NormLevels {
 // with 2^e > max, so that every term is below 1 (no FP32 overflow), per thread in
 // FP32 and across the CTA in FP64.  All levels in one launch: a launch per level
 // left the chip to 16 channels' fields at a time.
+template <int NL>
 __global__ void __launch_bounds__(kNormThreads)
-    k_field_norms(const __grid_constant__ NormLevels L, double *__restrict__ out) {
+    k_field_norms(const __grid_constant__ NormLevels<NL> L, double *__restrict__ out) {
   __shared__ float smax[kNormThreads / 32];
   __shared__ double s2s[kNormThreads / 32], s3s[kNormThreads / 32];
   __shared__ float bmax;
@@ -144,8 +147,9 @@ struct BoundLevel {
   double floor16;       // 2^-25 (2^14 + 2^7) M^2 (split FP16), else 0
 };
 
+template <int NL>
 struct BoundArgs {
-  BoundLevel lev[kMaxLevels];
+  BoundLevel lev[NL];
   int nc, ntrip;
   int batch;            // realisations written (the caller's, or internal for mode 2)
   int mode;             // 0 bound of S / (A M^2 T); 1 general plan: four evaluations per
@@ -154,17 +158,21 @@ struct BoundArgs {
 };
 
 // First-order bound on |dS| of one real evaluation (internal realisation b) of
-// the ring triple with rings r.  Called by a whole warp, the lanes over the
-// channels: the norms are the largest over each ring's fields.
+// the ring triple with rings r, in lane 0.  Called by a whole warp, the lanes over the
+// channels: the norms are the largest over each ring's fields (of nc < 17 channels
+// only the first lanes hold any: the exchange starts at the half of their power of two;
+// from 16 on, 4 channels took 1.7 us more than a thread each).
 __device__ double trip_beta(const BoundLevel &L, int nc, int b, const int r[3]) {
   double nm[3][3];  // [ring][max, 2-norm, 3-norm]
+  int o0 = 16;
+  while (o0 >= nc) o0 >>= 1;
   for (int q = 0; q < 3; ++q) {
     const double *n = L.norms + ((long long)b * L.nslot + L.slot_of[r[q]]) * nc * 3;
     for (int k = 0; k < 3; ++k) nm[q][k] = 0.0;
     for (int c = threadIdx.x & 31; c < nc; c += 32)
       for (int k = 0; k < 3; ++k) nm[q][k] = fmax(nm[q][k], n[3 * c + k]);
     for (int k = 0; k < 3; ++k)
-      for (int o = 16; o; o >>= 1)
+      for (int o = o0; o; o >>= 1)
         nm[q][k] = fmax(nm[q][k], __shfl_xor_sync(0xffffffffu, nm[q][k], o));
   }
   double fft = 0.0;
@@ -184,7 +192,8 @@ __device__ double trip_beta(const BoundLevel &L, int nc, int b, const int r[3]) 
 // bound[b][trip] of every ring triple (table: i, j, l, level), a warp each.  One
 // thread each walked nine dependent rows of norms per ring triple, a launch per level:
 // 12 us each for 16 channels.
-__global__ void k_trip_bound(const __grid_constant__ BoundArgs A, const int *__restrict__ tab,
+template <int NL>
+__global__ void k_trip_bound(const __grid_constant__ BoundArgs<NL> A, const int *__restrict__ tab,
                              const double *__restrict__ tnorm, double *__restrict__ bound) {
   const int t = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   if (t >= A.batch * A.ntrip) return;
@@ -268,6 +277,55 @@ int ceil_log2(int m) {
   return k;
 }
 
+// Field norms and ring-triple bounds of a plan of at most NL image sides.
+struct BoundJob {
+  int batch, mode;  // of BoundArgs
+  double c_term;
+  const int *tab;   // device: ring triples (i, j, l, level)
+  double *bound;    // device
+};
+template <int NL>
+cudaError_t launch_trip_bound(bs_plan p, const BoundJob &job, cudaStream_t s) {
+  const int prec = p->d.precision;
+  double *norms = p->at<double>(p->L.errn);
+  NormLevels<NL> N{};
+  BoundArgs<NL> B{};
+  B.nc = p->nc;
+  B.batch = job.batch;
+  B.mode = job.mode;
+  B.ntrip = p->ntrip;
+  const int nlev = (int)p->levels.size();
+  for (int li = 0; li < nlev; ++li) {
+    const Level &lv = p->levels[li];
+    const long long m2 = (long long)lv.M * lv.M;
+    const int nfield = p->batch * lv.nslot * p->nc;
+    N.F[li] = p->at<float>(lv.offF);
+    N.m2[li] = m2;
+    N.first[li + 1] = N.first[li] + nfield;
+    BoundLevel &L = B.lev[li];
+    L.norms = norms + (size_t)N.first[li] * 3;
+    L.slot_of = p->at<int>(lv.offSlot);
+    L.kexp = prec == BS_PREC_SPLIT_FP16 ? p->at<int>(lv.offKexp) : nullptr;
+    L.nslot = lv.nslot;
+    const double c_acc = prec == BS_PREC_FP32
+                             ? (1024.0 + std::ceil((double)m2 / 1024.0) + 1.0) * kU
+                             : 2.0 * kU * (3.0 * std::ceil((double)m2 / 16.0) + 1.0);
+    L.c1 = job.c_term + c_acc;
+    L.cf = (2.0 * (ceil_log2(lv.M) + 2) * 8.0 + 2.0) * kU;
+    L.floor16 = prec == BS_PREC_SPLIT_FP16 ? std::ldexp(1.0, -25) * (16384.0 + 128.0) * (double)m2
+                                           : 0.0;
+  }
+  const int nfields = N.first[nlev];
+  if (nfields == 0) return cudaSuccess;
+  k_field_norms<NL><<<nfields, kNormThreads, 0, s>>>(N, norms);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const long long nt = 32LL * B.batch * p->ntrip;
+  k_trip_bound<NL><<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(B, job.tab, p->at<double>(p->L.tnorm),
+                                                                job.bound);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 }  // namespace bsi
@@ -320,42 +378,10 @@ extern "C" bs_status bs_mabs_error_bound(bs_plan p, double *bound_dev, const dou
   }
   // NaN (all bits set) for every ring triple without a closed triangle
   EB_CUDA(cudaMemsetAsync(bound_dev, 0xFF, (size_t)out_batch * p->ntrip * sizeof(double), s));
-  double *norms = p->at<double>(p->L.errn);
-  NormLevels N{};
-  BoundArgs B{};
-  B.nc = p->nc;
-  B.batch = p->chans ? p->batch : out_batch;
-  B.mode = p->chans ? 2 : p->general ? 1 : 0;
-  B.ntrip = p->ntrip;
-  for (int li = 0; li < (int)p->levels.size(); ++li) {
-    const Level &lv = p->levels[li];
-    const long long m2 = (long long)lv.M * lv.M;
-    const int nfield = p->batch * lv.nslot * p->nc;
-    N.F[li] = p->at<float>(lv.offF);
-    N.m2[li] = m2;
-    N.first[li + 1] = N.first[li] + nfield;
-    BoundLevel &L = B.lev[li];
-    L.norms = norms + (size_t)N.first[li] * 3;
-    L.slot_of = p->at<int>(lv.offSlot);
-    L.kexp = prec == BS_PREC_SPLIT_FP16 ? p->at<int>(lv.offKexp) : nullptr;
-    L.nslot = lv.nslot;
-    const double c_acc = prec == BS_PREC_FP32
-                             ? (1024.0 + std::ceil((double)m2 / 1024.0) + 1.0) * kU
-                             : 2.0 * kU * (3.0 * std::ceil((double)m2 / 16.0) + 1.0);
-    L.c1 = c_term + c_acc;
-    L.cf = (2.0 * (ceil_log2(lv.M) + 2) * 8.0 + 2.0) * kU;
-    L.floor16 = prec == BS_PREC_SPLIT_FP16 ? std::ldexp(1.0, -25) * (16384.0 + 128.0) * (double)m2
-                                           : 0.0;
-  }
-  const int nfields = N.first[p->levels.size()];
-  if (nfields > 0) {
-    k_field_norms<<<nfields, kNormThreads, 0, s>>>(N, norms);
-    EB_CUDA(cudaGetLastError());
-    const long long nt = 32LL * B.batch * p->ntrip;
-    k_trip_bound<<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(B, dtab, p->at<double>(p->L.tnorm),
-                                                              p->chans ? beta_int : bound_dev);
-    EB_CUDA(cudaGetLastError());
-  }
+  const BoundJob job{p->chans ? p->batch : out_batch, p->chans ? 2 : p->general ? 1 : 0, c_term, dtab,
+                     p->chans ? beta_int : bound_dev};
+  EB_CUDA(p->levels.size() == 1 ? launch_trip_bound<1>(p, job, s)
+                                : launch_trip_bound<kMaxLevels>(p, job, s));
   if (p->chans) {
     const int npl = closable ? (int)p->clos.size() : p->ntrip;
     const long long n2 = (long long)(2 * p->nc - 1) * (2 * p->nc - 1);

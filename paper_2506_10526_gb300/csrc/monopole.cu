@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kThreads) k_mono_bins(const MonoArgs a, long l
 // own, all at once: with narrow bins every lane closes another bin on every row.  Bin
 // after bin through the shuffles, 170 planes of 32^2 in 40 x 10 x 10 bins, four
 // realisations, took 387 us against 104 of the row walk; 79 now (calls, with their
-// launches; more than two lanes instead of eight: 90).
+// launches; more than two lanes instead of eight: 91).
 template <int NX>
 __device__ __forceinline__ void flush_lanes(unsigned who, int cur, const double *x, unsigned cnt,
                                             int nx, int nbin, double *hs, unsigned *hc, int lane) {
