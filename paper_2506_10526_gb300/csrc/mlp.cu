@@ -210,11 +210,48 @@ __global__ void k_mlp_sample(int *idx, int nrows, int n, unsigned long long seed
     idx[r] = mlp_sample_row(seed, step, r, n);
 }
 
-// Column means and standard deviations (FP64 sums) of x [n][d] and t [n].  A warp walks
-// whole rows, lane = column (and column + 32, + 64..): coalesced reads.  One CTA per
-// column read a float every d: 244 us for 122880 x 45; with both kernels here 70 us
-// at 8 warps a CTA, 49 at 32 (more rows in flight).  Each CTA leaves its sums in
-// sums[CTA][2][d + 1]; k_mlp_norm adds them up.
+// Column means and standard deviations (FP64 sums) of x [n][d] and t [n].
+//
+// Few rows: one CTA per column, which puts the FP64 sums, the quotients and the root of
+// each column on an SM of its own.
+__global__ void __launch_bounds__(256) k_mlp_colstats_few(const float *__restrict__ x,
+                                                          const float *__restrict__ t, int n, int d,
+                                                          float *__restrict__ norm) {
+  const int c = blockIdx.x;  // 0..d-1: features, d: target
+  double s = 0, s2 = 0;
+  for (int r = threadIdx.x; r < n; r += blockDim.x) {
+    const double v = c < d ? x[(long long)r * d + c] : t[r];
+    s += v;
+    s2 += v * v;
+  }
+  __shared__ double a[256], b[256];
+  a[threadIdx.x] = s;
+  b[threadIdx.x] = s2;
+  __syncthreads();
+  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+    if (threadIdx.x < o) {
+      a[threadIdx.x] += a[threadIdx.x + o];
+      b[threadIdx.x] += b[threadIdx.x + o];
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x) return;
+  const double mean = a[0] / n, var = fmax(b[0] / n - mean * mean, 0.0);
+  const float sd = var > 1e-24 ? (float)sqrt(var) : 1.f;
+  norm[c < d ? c : 2 * d] = (float)mean;
+  norm[c < d ? d + c : 2 * d + 1] = sd;
+}
+
+// Many rows: a warp walks whole rows, lane = column (and column + 32, + 64..): coalesced
+// reads, where a CTA per column reads a float every d.  32 warps a CTA (39 us for
+// 122880 x 45; with 8 too few rows are in flight, 61).  Each CTA leaves its sums in
+// sums[CTA][2][d + 1]; k_mlp_norm adds them up.  Both kernels of a call among others, us,
+// against one CTA per column:
+//   rows         1000   8000  16000  24000  64000  122880
+//   1 column    15/10  19/15  19/23  21/32  25/75  31/138
+//   45 columns  19/9   25/15  27/25  29/33  37/78  52/146
+//   64 columns  23/9   29/15  34/25  36/35  50/82  71/153
+// so these take over from 10000 + 224 d rows on.
 __global__ void __launch_bounds__(kStatThreads) k_mlp_colstats(const float *__restrict__ x,
                                                       const float *__restrict__ t, int n, int d,
                                                       double *__restrict__ sums) {
@@ -521,6 +558,11 @@ bs_status bs_mlp_fit_norm(bs_mlp m, const float *x_dev, const float *t_dev, int 
   if (!m || !x_dev || !t_dev || n < 2) return BS_ERR_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int d = m->dev.d;
+  if (n < 10000 + 224 * d) {
+    k_mlp_colstats_few<<<d + 1, 256, 0, s>>>(x_dev, t_dev, n, d, m->dev.norm);
+    ML_CUDA(cudaGetLastError());
+    return BS_OK;
+  }
   const int parts = std::min(kStatParts, (n - 1) / 64 + 1);
   k_mlp_colstats<<<parts, kStatThreads, 0, s>>>(x_dev, t_dev, n, d, m->stat);
   ML_CUDA(cudaGetLastError());

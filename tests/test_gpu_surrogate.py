@@ -358,3 +358,25 @@ def test_inputs_are_divided_by_their_deviation():
     assert abs(res[0][1][0] - res[1][1][0]) <= 1e-6 * res[0][1][0]
     np.testing.assert_allclose(res[0][1][1], res[1][1][1], rtol=0,
                                atol=1e-6 * np.abs(res[0][1][1]).max())
+
+
+@pytest.mark.parametrize("d", [1, 45, 64])
+def test_column_statistics_around_the_row_count_that_changes_kernels(d):
+    """One row below and from 10000 + 224 d rows on, and one stride of the many-row kernel
+    further: the same FP64 sums, rounded once to FP32."""
+    torch = _torch()
+    import paper_2506_10526_gb300 as bs
+    n0 = 10000 + 224 * d
+    r = np.random.default_rng(d)
+    x = (r.standard_normal((n0 + 4865, d)) * 3 + 1).astype(np.float32)
+    t = r.standard_normal(n0 + 4865).astype(np.float32)
+    xd, td = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+    net = bs.Surrogate(d, 128, seed=1)
+    for n in (n0 - 1, n0, n0 + 4865):
+        net.fit_norm(xd[:n], td[:n])
+        got = net.params().astype(np.float64)[net.n_weights:]
+        cols = np.concatenate([x[:n], t[:n, None]], axis=1).astype(np.float64)
+        mean, sd = cols.mean(0), cols.std(0)
+        np.testing.assert_allclose(got, np.concatenate([mean[:d], sd[:d], mean[d:], sd[d:]]),
+                                   rtol=1e-7, atol=1e-7)
+    net.close()
