@@ -150,7 +150,7 @@ struct BoundLevel {
 template <int NL>
 struct BoundArgs {
   BoundLevel lev[NL];
-  int nc, ntrip;
+  int nc, ntrip, lanes;
   int batch;            // realisations written (the caller's, or internal for mode 2)
   int mode;             // 0 bound of S / (A M^2 T); 1 general plan: four evaluations per
                         // realisation (t = 0, 1, -1, 2); 2 bound of each internal
@@ -158,22 +158,20 @@ struct BoundArgs {
 };
 
 // First-order bound on |dS| of one real evaluation (internal realisation b) of
-// the ring triple with rings r, in lane 0.  Called by a whole warp, the lanes over the
-// channels: the norms are the largest over each ring's fields (of nc < 17 channels
-// only the first lanes hold any: the exchange starts at the half of their power of two;
-// from 16 on, 4 channels took 1.7 us more than a thread each).
-__device__ double trip_beta(const BoundLevel &L, int nc, int b, const int r[3]) {
+// the ring triple with rings r.  Called by `lanes` neighbouring threads (a power of two,
+// `mask` of their warp's), over the channels: the norms are the largest over each
+// ring's fields.
+__device__ double trip_beta(const BoundLevel &L, int nc, int b, const int r[3], int lanes,
+                            unsigned mask) {
   double nm[3][3];  // [ring][max, 2-norm, 3-norm]
-  int o0 = 16;
-  while (o0 >= nc) o0 >>= 1;
   for (int q = 0; q < 3; ++q) {
     const double *n = L.norms + ((long long)b * L.nslot + L.slot_of[r[q]]) * nc * 3;
     for (int k = 0; k < 3; ++k) nm[q][k] = 0.0;
-    for (int c = threadIdx.x & 31; c < nc; c += 32)
+    for (int c = threadIdx.x & (lanes - 1); c < nc; c += lanes)
       for (int k = 0; k < 3; ++k) nm[q][k] = fmax(nm[q][k], n[3 * c + k]);
     for (int k = 0; k < 3; ++k)
-      for (int o = o0; o; o >>= 1)
-        nm[q][k] = fmax(nm[q][k], __shfl_xor_sync(0xffffffffu, nm[q][k], o));
+      for (int o = lanes >> 1; o; o >>= 1)
+        nm[q][k] = fmax(nm[q][k], __shfl_xor_sync(mask, nm[q][k], o));
   }
   double fft = 0.0;
   for (int q = 0; q < 3; ++q) {
@@ -189,13 +187,14 @@ __device__ double trip_beta(const BoundLevel &L, int nc, int b, const int r[3]) 
   return beta;
 }
 
-// bound[b][trip] of every ring triple (table: i, j, l, level), a warp each.  One
-// thread each walked nine dependent rows of norms per ring triple, a launch per level:
-// 12 us each for 16 channels.
+// bound[b][trip] of every ring triple (table: i, j, l, level), A.lanes threads each
+// (bound_lanes).
 template <int NL>
 __global__ void k_trip_bound(const __grid_constant__ BoundArgs<NL> A, const int *__restrict__ tab,
                              const double *__restrict__ tnorm, double *__restrict__ bound) {
-  const int t = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
+  const int lanes = A.lanes;
+  const int t = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) / lanes);
+  const unsigned mask = (0xffffffffu >> (32 - lanes)) << (threadIdx.x & 31 & ~(lanes - 1));
   if (t >= A.batch * A.ntrip) return;
   const int b = t / A.ntrip, trip = t - b * A.ntrip;
   if (tab[4 * trip + 3] < 0 || !(tnorm[trip] > 0.0)) return;
@@ -203,15 +202,15 @@ __global__ void k_trip_bound(const __grid_constant__ BoundArgs<NL> A, const int 
   const int r[3] = {tab[4 * trip], tab[4 * trip + 1], tab[4 * trip + 2]};
   double beta;
   if (A.mode != 1) {
-    beta = trip_beta(L, A.nc, b, r);
+    beta = trip_beta(L, A.nc, b, r, lanes, mask);
   } else {  // evaluations t = 0, 1, -1, 2 of realisation b are internal 4b .. 4b + 3
-    const double b0 = trip_beta(L, A.nc, 4 * b, r), b1 = trip_beta(L, A.nc, 4 * b + 1, r),
-                 bm = trip_beta(L, A.nc, 4 * b + 2, r), b2 = trip_beta(L, A.nc, 4 * b + 3, r);
+    const double b0 = trip_beta(L, A.nc, 4 * b, r, lanes, mask), b1 = trip_beta(L, A.nc, 4 * b + 1, r, lanes, mask),
+                 bm = trip_beta(L, A.nc, 4 * b + 2, r, lanes, mask), b2 = trip_beta(L, A.nc, 4 * b + 3, r, lanes, mask);
     const double re = 2.0 * b0 + 0.5 * (b1 + bm);
     const double im = (9.0 * b1 + bm + 2.0 * b2 + 6.0 * b0) / 6.0;
     beta = sqrt(re * re + im * im);
   }
-  if ((threadIdx.x & 31) == 0)
+  if ((threadIdx.x & (lanes - 1)) == 0)
     bound[(long long)b * A.ntrip + trip] = A.mode == 2 ? 1.01 * beta : 1.01 * beta * tnorm[trip];
 }
 
@@ -277,6 +276,21 @@ int ceil_log2(int m) {
   return k;
 }
 
+// Threads per ring triple of k_trip_bound: the power of two that covers the channels, at
+// most a warp, while the triples together keep within 8 warps an SM.  FP64 issue
+// bounds the kernel: a warp per triple spends 9 maxima over five exchanges on each,
+// which for many triples costs more than a thread's walk over the channels of its nine
+// norms; that walk is one long chain where there are few.  us, a thread per triple / a
+// warp / this: 20 triples of 4 channels 5.9 / 7.5 / 5.9, 220 of 16 channels (on six sides,
+// a launch each with a thread) 70 / 7.9 / 7.9, 20 of 256 channels 139 / 12.3 / 13.0, 8 x 1540
+// of 13 channels 13 / 50 / 11, 8 x 2600 of 16 channels 16.3 / 70 / 16.8 (with 4 or 16 warps
+// an SM 11 to 13 and 13 to 18 where this takes 9 to 17).
+int bound_lanes(int nc, long long ntriples) {
+  int lanes = 1;
+  while (lanes < 32 && lanes < nc && 2 * lanes * ntriples <= 152LL * 8 * 32) lanes *= 2;
+  return lanes;
+}
+
 // Field norms and ring-triple bounds of a plan of at most NL image sides.
 struct BoundJob {
   int batch, mode;  // of BoundArgs
@@ -320,7 +334,8 @@ cudaError_t launch_trip_bound(bs_plan p, const BoundJob &job, cudaStream_t s) {
   k_field_norms<NL><<<nfields, kNormThreads, 0, s>>>(N, norms);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const long long nt = 32LL * B.batch * p->ntrip;
+  B.lanes = bound_lanes(p->nc, (long long)B.batch * p->ntrip);
+  const long long nt = (long long)B.lanes * B.batch * p->ntrip;
   k_trip_bound<NL><<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(B, job.tab, p->at<double>(p->L.tnorm),
                                                                 job.bound);
   return cudaGetLastError();

@@ -250,3 +250,27 @@ def test_bound_covers_the_error_per_channel_sampling(precision, multires):
         print(f"per-channel p{precision} mr{int(multires)} realisation {b}: error/bound max "
               f"{ratio.max():.2e} median {np.median(ratio):.2e}; infinite bins "
               f"{int(np.isinf(ebin[ok]).sum())} of {int(ok.sum())}")
+
+
+@pytest.mark.parametrize("nc,general", [(1, False), (9, False), (33, False), (9, True)])
+def test_bound_does_not_depend_on_the_threads_per_triple(nc, general):
+    """A realisation's bound in plans of 1, 6 and 48 realisations of 364 ring triples: 1 to
+    32 threads share a triple, and only maxima are shared, so the bounds are the same
+    bits."""
+    torch = _torch()
+    import paper_2506_10526_gb300 as bs
+    nt, edges = 16, np.linspace(0.9, 7.6, 13)
+    vis = np.stack([synth.sky_visibilities(nt, nc, seed=90 + k) for k in range(3)])
+    got = []
+    for batch in (1, 6, 48):
+        plan = bs.Plan(nt, nc, edges, batch=batch, general=general)
+        v = vis[np.arange(batch) % 3]
+        plan.grid_load(torch.from_numpy(np.ascontiguousarray(v.astype(np.complex64))).cuda())
+        got.append(plan.error_bound()[0].cpu().numpy())
+        plan.close()
+    assert np.isfinite(got[0]).any()
+    for g in got[1:]:
+        for b in range(g.shape[0]):
+            if b % 3 == 0:
+                np.testing.assert_array_equal(g[b], got[0][0])
+            np.testing.assert_array_equal(g[b], g[b % 3])
