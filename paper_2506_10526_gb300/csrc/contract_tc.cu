@@ -616,9 +616,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
       const int dmax = t.diag ? t.nu2_0 - t.nu1_0 : P1;
       const bool fast = use_red && G.out_full == nullptr;  // collapse only: shared reduction
       // the warps take each chunk together: the FP32 terms of an entry that lie in
-      // different warps are then added in the order of their chunks, run after run
-      // (free-running, a run's collapse differs from the next by 1e-8, the next run's
-      // 3D bispectrum variance by up to 1e-8; in step, not at all on most planes).
+      // different chunks are then added in the order of the chunks, run after run; the
+      // warps still race within a chunk (free-running, a run's collapse differs from the
+      // next by 1e-8, the next run's 3D bispectrum variance by up to 1e-8; in step, not at
+      // all on most planes).
       // Eight barriers a tile cost nothing measurable (25.3 ms either way for two runs
       // of 10 realisations of three uneven grids), but tiles of a few stages, which
       // are all epilogue, are left free-running.

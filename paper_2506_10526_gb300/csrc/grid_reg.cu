@@ -13,7 +13,8 @@
 //   [realisation][field][pair] order (pairs of several fields for small
 //   sides).  Pass 1 reads G straight from global memory (the Hermitian mirror
 //   z(M - u) = conj A(u) + i conj B(u) built on the fly); pass 2 threads take
-//   output columns fastest, so the F and hi / lo stores are consecutive.
+//   output columns fastest.  F and hi / lo leave straight from there or as whole rows
+//   from the exchange tile, by side and output form (RowCfg).
 #include <cuda_bf16.h>
 
 #include "bs_internal.h"
