@@ -82,7 +82,7 @@ __device__ __forceinline__ void div_column(float mu, float sd, float &nmu, float
   k = max(-126, min(126, k));
   c = __uint_as_float((uint32_t)(127 - k) << 23);
   nmu = -mu;
-  ns = -(sd * c);
+  ns = isinf(sd) ? 0.f : -(sd * c);  // an infinite deviation: r = 0, quotients 0
   r = 1.f / (sd * c);
 }
 __device__ __forceinline__ void normalise_pair(float x0, float x1, const DivPair &t, float &u0,

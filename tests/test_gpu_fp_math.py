@@ -103,3 +103,13 @@ def test_reciprocal_square_root(fpm):
     assert fpm.fpm_rsqrt(s.ctypes.data_as(p), y.ctypes.data_as(p), s.size) == 0
     want = 1 / np.sqrt(s.astype(np.longdouble))
     assert np.abs(y / want - 1).max() < 2.0 ** -52
+
+
+def test_normalised_inputs_of_infinite_deviations(fpm):
+    """Quotients by an infinite deviation are zero, as by a division; the neighbouring
+    column is not touched."""
+    a = np.array([3.0, 5.0, 1.0, 1.0, np.inf, 2.0], np.float32)
+    got = np.empty(2, np.float32)
+    p = ctypes.POINTER(ctypes.c_float)
+    assert fpm.fpm_normalise(a.ctypes.data_as(p), got.ctypes.data_as(p), 1) == 0
+    np.testing.assert_array_equal(got, [0.0, 2.0])
