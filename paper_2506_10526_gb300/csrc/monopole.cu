@@ -66,7 +66,6 @@ struct MonoArgs {
   int nc, n_k1, n_mu, n_t, nbin;
   int chunk;             // rows of a summing warp's range (mono_split)
   int mirror;            // multipoles: kpar is antisymmetric, samples go in pairs
-  int model;
   double f2, p_amp, p_half;  // 2 f_NG, amplitude, p_index / 2
   double *sums;          // [batch_total][nbin]
   unsigned long long *cnt;  // [nbin], or null (counted by an earlier launch)
@@ -143,7 +142,7 @@ __global__ void __launch_bounds__(kThreads) k_mono_bins(const MonoArgs a, long l
 // for the whole warp, nearly every group of 32 samples was mixed where the bins
 // are narrow along b, and went sample by sample through FP64 shared-memory
 // atomics (compare-and-swap loops): 3.34 ms for 216 planes of 768^2 (12 x 5 x 5
-// bins) against 0.44 ms now, 2.8 TB/s of bins and values (the FP64 adds alone
+// bins) against 0.43 ms now, 2.9 TB/s of bins and values (the FP64 adds alone
 // take 0.24 ms).
 //
 // Adds x[0..NX) of the lanes in `who` (a ballot; each lane's own bin `cur`) to the
@@ -186,10 +185,13 @@ __device__ __forceinline__ void flush_lanes(unsigned who, int cur, const double 
   }
 }
 
-template <int NB>  // realisations per launch held in registers (a.nbatch <= NB)
+// NB: realisations per launch held in registers (a.nbatch <= NB).  MODEL: values from
+// Eq. (bsana) instead of b3d; its powers in the same kernel took registers and spilled
+// (684 planes of 768^2, few bins a plane: 1.12 ms, 0.88 without; the row walk 1.04).
+template <int NB, bool MODEL>
 __global__ void __launch_bounds__(kThreads) k_mono_sum(const MonoArgs a,
                                                        const int16_t *__restrict__ bins) {
-  constexpr int UR = NB == 1 ? 8 : NB == 2 ? 4 : 2;  // rows loaded ahead
+  constexpr int UR = NB <= 2 ? 4 : 2;  // rows loaded ahead
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double *hs = reinterpret_cast<double *>(smem_raw);                             // [nbatch][nbin]
   unsigned *hc = reinterpret_cast<unsigned *>(hs + (size_t)a.nbatch * a.nbin);  // [nbin]
@@ -197,7 +199,7 @@ __global__ void __launch_bounds__(kThreads) k_mono_sum(const MonoArgs a,
   for (int q = threadIdx.x; q < a.nbatch * a.nbin; q += blockDim.x) hs[q] = 0.0;
   for (int q = threadIdx.x; q < a.nbin; q += blockDim.x) hc[q] = 0u;
   __syncthreads();
-  const int nb = a.model ? 1 : a.nbatch;
+  const int nb = MODEL ? 1 : a.nbatch;
   const int i = a.rings[3 * p], j = a.rings[3 * p + 1], l = a.rings[3 * p + 2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int unit = blockIdx.x * (kThreads / 32) + warp, ncw = (a.nc + 31) / 32;
@@ -226,9 +228,9 @@ __global__ void __launch_bounds__(kThreads) k_mono_sum(const MonoArgs a,
       if (q[u] >= 0 && !BS_CHK(q[u], a.nbin, 41)) q[u] = -1;  // a bin outside the histogram
 #pragma unroll
       for (int b = 0; b < NB; ++b)
-        v[u][b] = (!a.model && b < nb && live) ? __ldg(vb + (long long)b * a.bstride + e) : 0.0;
+        v[u][b] = (!MODEL && b < nb && live) ? __ldg(vb + (long long)b * a.bstride + e) : 0.0;
     }
-    if (a.model) {
+    if constexpr (MODEL) {
 #pragma unroll
       for (int u = 0; u < UR; ++u)
         if (q[u] >= 0) v[u][0] = model_value(a, i, j, l, g0 + u, ib);
@@ -244,6 +246,7 @@ __global__ void __launch_bounds__(kThreads) k_mono_sum(const MonoArgs a,
 #pragma unroll
         for (int b = 0; b < NB; ++b) run[b] = 0.0;
       }
+      if (!__any_sync(0xffffffffu, cur >= 0)) continue;  // FP64 adds of dropped rows cost as much
       ++cnt;
 #pragma unroll
       for (int b = 0; b < NB; ++b)
@@ -709,15 +712,15 @@ bs_status bs_bs_monopole(bs_plan p, const double *b3d, const double *kperp_host,
   MONO_CUDA(cudaMemsetAsync(count_dev, 0, (size_t)nbin * sizeof(int64_t), s));
   const int npl = (int)p->clos.size();
   if (npl == 0) return BS_OK;
-  MONO_CUDA(smem_optin_once<k_mono_sum<1>>());
-  MONO_CUDA(smem_optin_once<k_mono_sum<2>>());
-  MONO_CUDA(smem_optin_once<k_mono_sum<4>>());
-  MONO_CUDA(smem_optin_once<k_mono_sum<kMaxBatch>>());
+  MONO_CUDA((smem_optin_once<k_mono_sum<1, true>>()));
+  MONO_CUDA((smem_optin_once<k_mono_sum<1, false>>()));
+  MONO_CUDA((smem_optin_once<k_mono_sum<2, false>>()));
+  MONO_CUDA((smem_optin_once<k_mono_sum<4, false>>()));
+  MONO_CUDA((smem_optin_once<k_mono_sum<kMaxBatch, false>>()));
   MonoArgs a{};
   a.b3d = b3d;
   st = mono_geometry(p, kperp_host, kpar_host, k1_edges_host, n_k1, n_mu, n_t, s, a);
   if (st != BS_OK) return st;
-  a.model = b3d ? 0 : 1;
   a.f2 = 2.0 * f_ng;
   a.p_amp = p_amp;
   a.p_half = 0.5 * p_index;
@@ -735,14 +738,16 @@ bs_status bs_bs_monopole(bs_plan p, const double *b3d, const double *kperp_host,
     if (b0 > 0) a.cnt = nullptr;  // the same samples: counted by the first launch
     const dim3 grid(gx, npl);
     const size_t sm = mono_smem(nbin, a.nbatch);
-    if (a.nbatch == 1)
-      k_mono_sum<1><<<grid, kThreads, sm, s>>>(a, p->mono_bins);
+    if (!b3d)
+      k_mono_sum<1, true><<<grid, kThreads, sm, s>>>(a, p->mono_bins);
+    else if (a.nbatch == 1)
+      k_mono_sum<1, false><<<grid, kThreads, sm, s>>>(a, p->mono_bins);
     else if (a.nbatch == 2)
-      k_mono_sum<2><<<grid, kThreads, sm, s>>>(a, p->mono_bins);
+      k_mono_sum<2, false><<<grid, kThreads, sm, s>>>(a, p->mono_bins);
     else if (a.nbatch <= 4)
-      k_mono_sum<4><<<grid, kThreads, sm, s>>>(a, p->mono_bins);
+      k_mono_sum<4, false><<<grid, kThreads, sm, s>>>(a, p->mono_bins);
     else
-      k_mono_sum<kMaxBatch><<<grid, kThreads, sm, s>>>(a, p->mono_bins);
+      k_mono_sum<kMaxBatch, false><<<grid, kThreads, sm, s>>>(a, p->mono_bins);
     MONO_CUDA(cudaGetLastError());
   }
   if (cplx) return join_general(p, a.sums, nbin, sum_dev, s);
