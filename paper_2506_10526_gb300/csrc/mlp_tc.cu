@@ -39,7 +39,9 @@ namespace {
 
 using fpm::DivPair;
 using fpm::normalise_pair;
+using fpm::scale_pair;
 using fpm::tanh_pair;
+using fpm::tanh_pair_grad;
 
 constexpr int W = 128;           // hidden width of the tensor-core kernels
 constexpr int kWarps = 8, kThreads = 32 * kWarps, kRowsPerCta = 16 * kWarps;
@@ -417,7 +419,7 @@ __global__ void __launch_bounds__(kGradThreads, 1)
       float v0 = 0.f, v1 = 0.f;
       if (row >= 0) {
         const float *xr = x + (long long)row * d;
-        normalise_pair(c < d ? xr[c] : 0.f, c + 1 < d ? xr[c + 1] : 0.f, norm[c / 2], v0, v1);
+        scale_pair(c < d ? xr[c] : 0.f, c + 1 < d ? xr[c + 1] : 0.f, norm[c / 2], v0, v1);
       }
       uint32_t hi, lo;
       split2(v0, v1, hi, lo);
@@ -470,8 +472,8 @@ __global__ void __launch_bounds__(kGradThreads, 1)
     };
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      tanh_pair(h1[j][0], h1[j][1], h1[j][0], h1[j][1]);
-      tanh_pair(h1[j][2], h1[j][3], h1[j][2], h1[j][3]);
+      tanh_pair_grad(h1[j][0], h1[j][1], h1[j][0], h1[j][1]);
+      tanh_pair_grad(h1[j][2], h1[j][3], h1[j][2], h1[j][3]);
       put(Ly::H1, j, h1[j]);
     }
     __syncthreads();
@@ -503,8 +505,8 @@ __global__ void __launch_bounds__(kGradThreads, 1)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const float2 w = *reinterpret_cast<const float2 *>(w3 + 32 * cq + 8 * j + 2 * t);
-      tanh_pair(c2[j][0], c2[j][1], c2[j][0], c2[j][1]);
-      tanh_pair(c2[j][2], c2[j][3], c2[j][2], c2[j][3]);
+      tanh_pair_grad(c2[j][0], c2[j][1], c2[j][0], c2[j][1]);
+      tanh_pair_grad(c2[j][2], c2[j][3], c2[j][2], c2[j][3]);
       y0 = fmaf(w.x, c2[j][0], fmaf(w.y, c2[j][1], y0));
       y1 = fmaf(w.x, c2[j][2], fmaf(w.y, c2[j][3], y1));
     }

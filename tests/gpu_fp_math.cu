@@ -8,23 +8,31 @@
 
 namespace {
 
-__global__ void k_tanh(const float *x, float *y, int n) {
+// kind 0: tanh_pair, 1: tanh_pair_grad
+__device__ void tanh_of(int kind, float x0, float x1, float &y0, float &y1) {
+  if (kind == 0)
+    bsi::fpm::tanh_pair(x0, x1, y0, y1);
+  else
+    bsi::fpm::tanh_pair_grad(x0, x1, y0, y1);
+}
+
+__global__ void k_tanh(int kind, const float *x, float *y, int n) {
   const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (i >= n) return;
   float y0, y1;
-  bsi::fpm::tanh_pair(x[i], i + 1 < n ? x[i + 1] : 0.f, y0, y1);
+  tanh_of(kind, x[i], i + 1 < n ? x[i + 1] : 0.f, y0, y1);
   y[i] = y0;
   if (i + 1 < n) y[i + 1] = y1;
 }
 
 // largest relative error of tanh over the n arguments with bit patterns lo, lo + 1, ..,
 // and the sum of the relative differences to the correctly rounded FP32 value
-__global__ void k_tanh_err(uint32_t lo, uint32_t n, unsigned long long *mx, double *sum) {
+__global__ void k_tanh_err(int kind, uint32_t lo, uint32_t n, unsigned long long *mx, double *sum) {
   double m = 0.0, s = 0.0;
   for (uint32_t i = 2 * (blockIdx.x * blockDim.x + threadIdx.x); i < n; i += 2 * gridDim.x * blockDim.x) {
     const float x0 = __uint_as_float(lo + i), x1 = -__uint_as_float(lo + min(i + 1, n - 1));
     float y0, y1;
-    bsi::fpm::tanh_pair(x0, x1, y0, y1);
+    tanh_of(kind, x0, x1, y0, y1);
     const double e0 = y0 / tanh((double)x0) - 1.0, e1 = y1 / tanh((double)x1) - 1.0;
     m = fmax(m, fmax(fabs(e0), fabs(e1)));
     const float r0 = (float)tanh((double)x0), r1 = (float)tanh((double)x1);
@@ -82,12 +90,12 @@ int fpm_normalise(const float *in, float *out, int n) {
 
 
 // y[n] = tanh(x[n]), host pointers
-int fpm_tanh(const float *x, float *y, int n) {
+int fpm_tanh(int kind, const float *x, float *y, int n) {
   float *d = nullptr;
   if (n < 1 || cudaMalloc(&d, 2 * (size_t)n * sizeof(float)) != cudaSuccess) return 1;
   cudaError_t e = cudaMemcpy(d, x, (size_t)n * sizeof(float), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
-    k_tanh<<<((n + 1) / 2 + 255) / 256, 256>>>(d, d + n, n);
+    k_tanh<<<((n + 1) / 2 + 255) / 256, 256>>>(kind, d, d + n, n);
     e = cudaMemcpy(y, d + n, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost);
   }
   cudaFree(d);
@@ -95,13 +103,13 @@ int fpm_tanh(const float *x, float *y, int n) {
 }
 
 // out: largest relative error, mean error
-int fpm_tanh_err(uint32_t lo, uint32_t n, double *out) {
+int fpm_tanh_err(int kind, uint32_t lo, uint32_t n, double *out) {
   double *d = nullptr;
   if (n < 1 || n > (1u << 30) || cudaMalloc(&d, 16) != cudaSuccess) return 1;
   double h[2] = {0.0, 0.0};
   cudaError_t e = cudaMemcpy(d, h, 16, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
-    k_tanh_err<<<152 * 8, 256>>>(lo, n, reinterpret_cast<unsigned long long *>(d), d + 1);
+    k_tanh_err<<<152 * 8, 256>>>(kind, lo, n, reinterpret_cast<unsigned long long *>(d), d + 1);
     e = cudaMemcpy(h, d, 16, cudaMemcpyDeviceToHost);
   }
   cudaFree(d);

@@ -31,40 +31,46 @@ def fpm(tmp_path_factory):
     return ctypes.CDLL(str(out))
 
 
-def _tanh(fpm, x):
+def _tanh(fpm, x, kind):
     x = np.ascontiguousarray(x, np.float32)
     y = np.empty_like(x)
     p = ctypes.POINTER(ctypes.c_float)
-    assert fpm.fpm_tanh(x.ctypes.data_as(p), y.ctypes.data_as(p), x.size) == 0
+    assert fpm.fpm_tanh(kind, x.ctypes.data_as(p), y.ctypes.data_as(p), x.size) == 0
     return y
 
 
+# of tanh_pair and tanh_pair_grad: the stated relative error and bias
+TANH = [(1.8e-7, 1e-8), (2.3e-7, 2e-8)]
+
+
+@pytest.mark.parametrize("kind", [0, 1])
 @pytest.mark.parametrize("exponent", range(-13, 4))
-def test_tanh_of_every_argument(fpm, exponent):
+def test_tanh_of_every_argument(fpm, exponent, kind):
     """Each binade from 2^-13 to 16, every FP32 value, both signs: within the stated
-    1.8e-7 relative of tanh, and against the correctly rounded value no bias above
-    1e-8 (rounding alone is biased near 2^-13, where tanh(x) lies just below x)."""
+    relative error of tanh, and against the correctly rounded value no bias above the
+    stated one (rounding alone is biased near 2^-13, where tanh(x) lies just below x)."""
     lo = (127 + exponent) << 23
     out = (ctypes.c_double * 2)()
-    assert fpm.fpm_tanh_err(ctypes.c_uint32(lo), ctypes.c_uint32(1 << 23), out) == 0
-    assert out[0] <= 1.8e-7
-    assert abs(out[1]) <= 1e-8
+    assert fpm.fpm_tanh_err(kind, ctypes.c_uint32(lo), ctypes.c_uint32(1 << 23), out) == 0
+    assert out[0] <= TANH[kind][0]
+    assert abs(out[1]) <= TANH[kind][1]
 
 
-def test_tanh_special_values(fpm):
+@pytest.mark.parametrize("kind", [0, 1])
+def test_tanh_special_values(fpm, kind):
     """Zeros with their sign, the smallest and small values (tanh(x) = x to rounding
     below 2^-13), values beyond 16, infinities, NaN, and an odd function."""
     inf, nan = np.float32(np.inf), np.float32(np.nan)
-    y = _tanh(fpm, [0.0, -0.0, inf, -inf, nan, 16.0, -1e30, 3e38])
+    y = _tanh(fpm, [0.0, -0.0, inf, -inf, nan, 16.0, -1e30, 3e38], kind)
     assert y[0] == 0 and not np.signbit(y[0]) and y[1] == 0 and np.signbit(y[1])
     assert y[2] == 1 and y[3] == -1 and np.isnan(y[4])
     np.testing.assert_array_equal(y[5:], [1, -1, 1])
     r = np.random.default_rng(1)
     x = r.integers(1, 114 << 23, 100001).astype(np.uint32).view(np.float32)  # up to 2^-13
-    np.testing.assert_allclose(_tanh(fpm, x).astype(np.float64), np.tanh(x.astype(np.float64)),
-                               rtol=1.8e-7, atol=0)
+    np.testing.assert_allclose(_tanh(fpm, x, kind).astype(np.float64), np.tanh(x.astype(np.float64)),
+                               rtol=TANH[kind][0], atol=0)
     x = np.concatenate([x, r.standard_normal(100001).astype(np.float32)])
-    np.testing.assert_array_equal(_tanh(fpm, -x), -_tanh(fpm, x))
+    np.testing.assert_array_equal(_tanh(fpm, -x, kind), -_tanh(fpm, x, kind))
 
 
 @pytest.mark.parametrize("spread", [1.0, 60.0, 126.0, 149.0])
